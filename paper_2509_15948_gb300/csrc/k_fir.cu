@@ -123,13 +123,55 @@ __global__ void __launch_bounds__(256) k_dly_fir(LaunchCtx c, const Item* __rest
 // update direction of z_m: sgn(g) + gamma (|z| - 1) z/|z| with
 //   g = sum_q G[q] conj(s'_q(z_hat)),  G[q] = sum_j dL/dh[m D + q + j] c_m[j],
 //   s'_q(z) = (1/D) [w^q (1 - z^D) - D z^{D-1} (1 - z w^q)] / (1 - z w^q)^2   (derivative of Eq. 18),
-// z_hat = z / max(1, |z|).  Near a pole (|1 - z w^q| < 1e-3) the series sum_k k a^{k-1} is summed directly.
+// z_hat = z / max(1, |z|).  Near a pole (a = z w^q, |1 - a| < 1e-3) the float quotient cancels, and
+// S = sum_{k=1}^{D-1} k a^{k-1} is evaluated in double (pole_sum).  What bounds the kernel: a block used to wait for
+// the one thread at the pole, whose D dependent double steps took 0.86 ms at D = 4410 (nearly all of the kernel's
+// time on a song of 16 tracks); its closed forms take a few microseconds.
+
+// S(a) = sum_{k=1}^{D-1} k a^{k-1} for a on or inside the unit circle, as D terms would give it in double.
+// With e = 1 - a: D |e| <= 6, the binomial series sum_j (-e)^j (j + 1) C(D, j + 2) (terms fall like (D |e|)^j / j!,
+// largest about 300 times the sum); beyond, (1 - a^{D-1} (1 + (D - 1) e)) / e^2, whose numerator no longer cancels.
+__device__ __noinline__ float2 pole_sum(float2 a, int D) {
+  const double er = 1.0 - (double)a.x, ei = -(double)a.y, dD = (double)D;
+  const double ee = er * er + ei * ei;
+  if (ee * dD * dD <= 36.0) {
+    double tr = 0.5 * dD * (dD - 1.0), ti = 0.0, sr = tr, si = 0.0;
+    const double stop = 1e-18 * tr;
+    for (int j = 0; j < 48; ++j) {   // t_{j+1} = -e t_j (j + 2) (D - j - 2) / ((j + 1) (j + 3))
+      const double r = -(dD - (double)(j + 2)) * ((double)(j + 2) / (double)((j + 1) * (j + 3)));
+      const double xr = (tr * er - ti * ei) * r, xi = (tr * ei + ti * er) * r;
+      tr = xr;
+      ti = xi;
+      sr += tr;
+      si += ti;
+      if (fabs(tr) + fabs(ti) < stop) break;
+    }
+    return make_float2((float)sr, (float)si);
+  }
+  double pr = 1.0, pi = 0.0, br = a.x, bi = a.y;   // a^{D-1} by squaring
+  for (int n = D - 1; n > 0; n >>= 1) {
+    if (n & 1) {
+      const double t = pr * br - pi * bi;
+      pi = pr * bi + pi * br;
+      pr = t;
+    }
+    const double t = br * br - bi * bi;
+    bi = 2.0 * br * bi;
+    br = t;
+  }
+  const double fr = 1.0 + (dD - 1.0) * er, fi = (dD - 1.0) * ei;
+  const double nr = 1.0 - (pr * fr - pi * fi), ni = -(pr * fi + pi * fr);
+  const double qr = er * er - ei * ei, qi = 2.0 * er * ei, k = 1.0 / (qr * qr + qi * qi);
+  return make_float2((float)((nr * qr + ni * qi) * k), (float)((ni * qr - nr * qi) * k));
+}
+
 __global__ void __launch_bounds__(256) k_dly_adj(LaunchCtx c, const Item* __restrict__ items) {
   __shared__ float cm[kDlyFir];
   __shared__ float dc[kDlyFir];
   __shared__ float red[2 * 32];
   __shared__ float gsum[2];
   __shared__ float2 zsh[3];   // z^D, z^(D-1), z clamped to the unit disk
+  __shared__ double zpow[6];  // cos, sin of D arg z and of (D - 1) arg z; |z|^D, |z|^(D-1)
   const Item it = items[blockIdx.x];
   const ProcDev& P = c.procs[it.proc];
   const int ch = it.idx / kDlyTaps, m = it.idx % kDlyTaps;
@@ -143,21 +185,26 @@ __global__ void __launch_bounds__(256) k_dly_adj(LaunchCtx c, const Item* __rest
     cm[threadIdx.x] = P.aux[(ch * kDlyTaps + m) * kDlyFir + threadIdx.x];
     dc[threadIdx.x] = dh[d + threadIdx.x];   // tap time d + j - 19 -> index d + j (first tap at -19)
   }
-  // (b, scalars) the powers of z in double, once per block (FP64 is slow; every thread used to repeat them)
-  if (threadIdx.x == 0) {
+  // (b, scalars) the powers of z in double, once per block, each factor on a warp of its own (FP64 is slow, and
+  // lanes of one warp would take their branches one after the other)
+  if ((threadIdx.x & 31) == 0 && threadIdx.x < 5 * 32) {
+    const int part = threadIdx.x >> 5;
     const double zr = pz[0], zi = pz[1];
     const double rz = sqrt(zr * zr + zi * zi);
     const double sc = rz > 1.0 ? 1.0 / rz : 1.0;
     const double hr = zr * sc, hi = zi * sc, hrad = rz * sc;
-    const double th = atan2(hi, hr);
-    double sD, cD, sD1, cD1;
-    sincos((double)D * th, &sD, &cD);
-    sincos((double)(D - 1) * th, &sD1, &cD1);
-    const double pD = hrad > 0.0 ? pow(hrad, (double)D) : 0.0;
-    const double pD1 = hrad > 0.0 ? pow(hrad, (double)(D - 1)) : 0.0;
-    zsh[0] = make_float2((float)(pD * cD), (float)(pD * sD));
-    zsh[1] = make_float2((float)(pD1 * cD1), (float)(pD1 * sD1));
-    zsh[2] = make_float2((float)hr, (float)hi);
+    if (part < 2) {
+      sincos((double)(D - part) * atan2(hi, hr), &zpow[2 * part + 1], &zpow[2 * part]);
+    } else if (part < 4) {
+      zpow[2 + part] = hrad > 0.0 ? pow(hrad, (double)(D - (part - 2))) : 0.0;
+    } else {
+      zsh[2] = make_float2((float)hr, (float)hi);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    const double r = zpow[4 + threadIdx.x];
+    zsh[threadIdx.x] = make_float2((float)(r * zpow[2 * threadIdx.x]), (float)(r * zpow[2 * threadIdx.x + 1]));
   }
   __syncthreads();
   // (a) log-magnitudes of c_m
@@ -188,16 +235,8 @@ __global__ void __launch_bounds__(256) k_dly_adj(LaunchCtx c, const Item* __rest
       const float2 den = cmul(oma, oma);
       const float dd = den.x * den.x + den.y * den.y;
       sp = cscale(cmulc(num, den), 1.f / ((float)D * dd));
-    } else {  // direct sum near the pole
-      double fr = 0.0, fi = 0.0;
-      const double ar = a.x, ai = a.y;
-      for (int k = D - 1; k >= 1; --k) {   // Horner: f = sum_{k=1}^{D-1} k a^{k-1}
-        const double nr = fr * ar - fi * ai + (double)k;
-        fi = fr * ai + fi * ar;
-        fr = nr;
-      }
-      const float2 f = make_float2((float)fr, (float)fi);
-      sp = cscale(cmul(wq, f), 1.f / (float)D);
+    } else {
+      sp = cscale(cmul(wq, pole_sum(a, D)), 1.f / (float)D);
     }
     accd[0] += (double)G * sp.x;   // g = sum G conj(s'), accumulated in double (|g| can be far below sum |G s'|)
     accd[1] -= (double)G * sp.y;
