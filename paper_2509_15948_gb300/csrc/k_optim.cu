@@ -6,87 +6,119 @@
 
 namespace mg {
 
-// One warp per processor: stats[0..1] = sums of the forward partials (LTI: E_ybar_mid, E_u_mid);
-// stats[4..11] = sums of the backward partials.
-__global__ void k_node_stats(LaunchCtx c, const int* __restrict__ procs, int n, int fwd) {
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (w >= n) return;
-  const ProcDev& P = c.procs[procs[w]];
-  if (lane >= kNPart) return;
+// Sum of a double over the block (blockDim.x a multiple of 32, at most 512) in a fixed order; every thread gets it.
+__device__ __forceinline__ double block_total(double v, double* red /* >= 16 */) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double s = 0.0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
+  return s;
+}
+
+// One CTA per processor: stats[0..1] = sums of the forward partials (LTI: E_ybar_mid, E_u_mid); stats[4..11] = sums
+// of the backward partials.  The rows (one per work item, up to about a thousand) are latency: 16 row groups of 8
+// columns read them side by side (with one group the kernel took 6-50 us per launch, waiting for one load after
+// the other; now 3-4 us).
+constexpr int kStatThreads = 128;
+__global__ void __launch_bounds__(kStatThreads) k_node_stats(LaunchCtx c, const int* __restrict__ procs, int fwd) {
+  __shared__ double part[kStatThreads / kNPart][kNPart];
+  const ProcDev& P = c.procs[procs[blockIdx.x]];
   const float* src = fwd ? P.fpart : P.bpart;
   const int rows = fwd ? P.nfpart : P.nbpart;
   if (src == nullptr) return;
+  const int col = threadIdx.x % kNPart, grp = threadIdx.x / kNPart;
+  constexpr int kGroups = kStatThreads / kNPart;
   double s = 0.0;
-  for (int r = 0; r < rows; ++r) s += (double)src[(size_t)r * kNPart + lane];
+#pragma unroll 4
+  for (int r = grp; r < rows; r += kGroups) s += (double)src[(size_t)r * kNPart + col];
+  part[grp][col] = s;
+  __syncthreads();
+  if (grp != 0) return;
+#pragma unroll
+  for (int g = 1; g < kGroups; ++g) s += part[g][col];
   if (fwd) {
-    if (lane < 2) P.stats[lane] = (float)s;
+    if (col < 2) P.stats[col] = (float)s;
   } else {
-    P.stats[4 + lane] = (float)s;
+    P.stats[4 + col] = (float)s;
   }
 }
 
 // One CTA per song.  mode 0: squared norms of the target spectrograms; mode 1: losses, backward
 // coefficients and the gain-staging coefficients of every LTI node; mode 2: L_a only (pruning trials).
-__global__ void __launch_bounds__(64) k_loss_finalize(LaunchCtx c, const SongDev* __restrict__ songs,
-                                                      const LossRes* __restrict__ resv, int nres,
-                                                      const float* __restrict__ alphas, int mode,
-                                                      float* out_losses, float* out_la, int la_stride) {
-  __shared__ double sums[3][6];
+// Latency-bound: a warp per (resolution, sum) adds the work items' partials, a thread per (resolution, set) forms the
+// loss terms, a thread per processor its regularisers.  (One thread going through items, terms and processors in turn
+// took 134 us on a song of 5 chains, 476 us on 20 and 748 us on 40: double-precision logarithms and dependent loads.)
+constexpr int kFinThreads = 256;
+__global__ void __launch_bounds__(kFinThreads) k_loss_finalize(LaunchCtx c, const SongDev* __restrict__ songs,
+                                                               const LossRes* __restrict__ resv, int nres,
+                                                               const float* __restrict__ alphas, int mode,
+                                                               float* out_losses, float* out_la, int la_stride) {
+  __shared__ double sums[3][6], term[3][3], red[16];
   const int si = blockIdx.x;
   const SongDev& S = songs[si];
-  const int t = threadIdx.x;
-  if (t < nres * 6) {
-    const int r = t / 6, j = t % 6;
+  const int t = threadIdx.x, lane = t & 31;
+  for (int p = t >> 5; p < nres * 6; p += kFinThreads / 32) {
+    const int r = p / 6, j = p % 6;
     double s = 0.0;
-    for (int i = 0; i < S.litems[r]; ++i) s += (double)S.lpart[((size_t)r * S.lcap + i) * 6 + j];
-    sums[r][j] = s;
+#pragma unroll 4
+    for (int i = lane; i < S.litems[r]; i += 32) s += (double)S.lpart[((size_t)r * S.lcap + i) * 6 + j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) sums[r][j] = s;
   }
   __syncthreads();
-  if (t != 0) return;
   if (mode == 0) {
-    for (int r = 0; r < nres; ++r)
-      for (int k = 0; k < 3; ++k) S.ynorm2[r * 3 + k] = sums[r][k];
+    if (t < nres * 3) S.ynorm2[t] = sums[t / 3][t % 3];
     return;
   }
-  double Lset[3] = {0.0, 0.0, 0.0};
-  for (int r = 0; r < nres; ++r) {
+  if (t < nres * 3) {
+    const int r = t / 3, k = t % 3;
     const int frames = S.nframes[r] - S.first_frame[r];
-    if (frames <= 0) {
-      for (int k = 0; k < 6; ++k) S.coef[r * 6 + k] = 0.f;
-      continue;
-    }
-    for (int k = 0; k < 3; ++k) {
+    double v = 0.0;
+    float c0 = 0.f, c1 = 0.f;
+    if (frames > 0) {
       const double cnt = (double)frames * resv[r].nbands * (k == 0 ? 2 : 1);
       const double yn = sqrt(S.ynorm2[r * 3 + k]);
       const double dn = sqrt(sums[r][2 * k + 1]);
-      Lset[k] += sums[r][2 * k] / cnt + dn / yn;
-      S.coef[r * 6 + 2 * k] = (float)(alphas[k] / cnt);
-      S.coef[r * 6 + 2 * k + 1] = dn > 0.0 ? (float)(alphas[k] / (dn * yn)) : 0.f;
+      v = sums[r][2 * k] / cnt + dn / yn;
+      c0 = (float)(alphas[k] / cnt);
+      c1 = dn > 0.0 ? (float)(alphas[k] / (dn * yn)) : 0.f;
     }
+    term[r][k] = v;
+    S.coef[r * 6 + 2 * k] = c0;
+    S.coef[r * 6 + 2 * k + 1] = c1;
   }
+  __syncthreads();
+  double Lset[3] = {0.0, 0.0, 0.0};
+  for (int r = 0; r < nres; ++r)
+    for (int k = 0; k < 3; ++k) Lset[k] += term[r][k];
   const double La = alphas[0] * Lset[0] + alphas[1] * Lset[1] + alphas[2] * Lset[2];
   if (mode == 2) {
-    out_la[si * la_stride] = (float)La;
+    if (t == 0) out_la[si * la_stride] = (float)La;
     return;
   }
-  double Lg = 0.0, Lp = 0.0;
-  for (int i = S.pbeg; i < S.pend; ++i) {
+  double lg = 0.0, lp = 0.0;
+  for (int i = S.pbeg + t; i < S.pend; i += kFinThreads) {
     const ProcDev& P = c.procs[i];
     if (!P.present) continue;
     double w = 1.0 / (1.0 + exp(-(double)c.q[P.qidx]));
     if (c.mask) w *= (double)c.mask[P.qidx];
-    Lp += w;
+    lp += w;
     if (P.type == T_E || P.type == T_R || P.type == T_D) {
       const double ey = P.stats[0], eu = P.stats[1];
       const double d = 0.5 * log(ey + 1e-12) - 0.5 * log(eu + 1e-12);
-      Lg += fabs(d);
+      lg += fabs(d);
       const double sg = d > 0.0 ? 1.0 : (d < 0.0 ? -1.0 : 0.0);
       P.stats[2] = (float)(c.alpha_g * sg / (ey + 1e-12));
       P.stats[3] = (float)(-c.alpha_g * sg / (eu + 1e-12));
     }
   }
-  const double ap = c.hyper[0];
-  if (out_losses) {
+  const double Lg = block_total(lg, red), Lp = block_total(lp, red);
+  if (t == 0 && out_losses) {
+    const double ap = c.hyper[0];
     float* o = out_losses + si * 7;
     o[0] = (float)La;
     o[1] = (float)Lset[0];
@@ -169,11 +201,11 @@ __global__ void k_set_hyper(float* hyper, float a0, float a1, float a2, float a3
 }
 
 void launch_node_stats(const LaunchCtx& c, const int* procs, int n, int fwd) {
-  if (n) k_node_stats<<<(n * 32 + 255) / 256, 256, 0, c.stream>>>(c, procs, n, fwd);
+  if (n) k_node_stats<<<n, kStatThreads, 0, c.stream>>>(c, procs, fwd);
 }
 void launch_loss_finalize_mode(const LaunchCtx& c, const SongDev* songs, int nsongs, const LossRes* res, int nres,
                                const float* alphas, int mode, float* out_losses, float* out_la, int la_stride) {
-  if (nsongs) k_loss_finalize<<<nsongs, 64, 0, c.stream>>>(c, songs, res, nres, alphas, mode, out_losses, out_la, la_stride);
+  if (nsongs) k_loss_finalize<<<nsongs, kFinThreads, 0, c.stream>>>(c, songs, res, nres, alphas, mode, out_losses, out_la, la_stride);
 }
 void launch_grad_finalize2(const LaunchCtx& c, const int* procs, int n, float* gq) {
   if (n) k_grad_finalize<<<(n + 127) / 128, 128, 0, c.stream>>>(c, procs, n, gq);
