@@ -218,10 +218,14 @@ struct mg_console {
   ProcList all_lti_present;
   DevVec<int4> loss_items[3];
   ItemList gather_items;
-  // evaluation metrics (Sec. 5.3): (song, 8 s segment) items, per-song item ranges, Bark band bin ranges
+  // evaluation metrics (Sec. 5.3): (song, 8 s segment) items, per-song item ranges, the work items of every segment's
+  // pieces (song, segment, 2 piece + signal) with per-segment ranges, Bark band bin ranges
   std::vector<int2> ev_items;
-  std::vector<int> ev_begin, ev_lo, ev_hi;
+  std::vector<int4> ev_parts;
+  std::vector<int> ev_begin, ev_pbegin, ev_lo, ev_hi;
   int2* d_ev_items = nullptr;
+  int4* d_ev_parts = nullptr;
+  int* d_ev_pbegin = nullptr;
   int* d_ev_begin = nullptr;
   int* d_ev_lo = nullptr;
   int* d_ev_hi = nullptr;
@@ -1905,14 +1909,23 @@ mg_status create_impl(mg_console* c, const mg_console_desc* d, const mg_song_des
                                      2700, 3150, 3700, 4400, 5300, 6400, 7700, 9500, 12000, 15500};
     c->ev_seg_len = (int)std::llround(8.0 * fs);
     c->ev_items.clear();
+    c->ev_parts.clear();
     c->ev_begin.clear();
+    c->ev_pbegin.clear();
     for (size_t si = 0; si < c->songs.size(); ++si) {
       c->ev_begin.push_back((int)c->ev_items.size());
       const int L = c->songs[si].L;
       const int nseg = L < c->ev_seg_len ? 1 : L / c->ev_seg_len;
-      for (int k = 0; k < nseg; ++k) c->ev_items.push_back(make_int2((int)si, k));
+      for (int k = 0; k < nseg; ++k) {
+        c->ev_items.push_back(make_int2((int)si, k));
+        c->ev_pbegin.push_back((int)c->ev_parts.size());
+        const int len = k == nseg - 1 ? L - k * c->ev_seg_len : c->ev_seg_len;   // the last one to the song's end
+        for (int p = 0; p < (len + kEvalPiece - 1) / kEvalPiece; ++p)
+          for (int h = 0; h < 2; ++h) c->ev_parts.push_back(make_int4((int)si, k, 2 * p + h, 0));
+      }
     }
     c->ev_begin.push_back((int)c->ev_items.size());
+    c->ev_pbegin.push_back((int)c->ev_parts.size());
     c->ev_lo.assign(24, 0);
     c->ev_hi.assign(24, 0);
     for (int b = 0; b < 24; ++b) {
@@ -1929,9 +1942,10 @@ mg_status create_impl(mg_console* c, const mg_console_desc* d, const mg_song_des
       c->ev_hi[b] = hi;
     }
     if (upload(c, c->ev_items, &c->d_ev_items) || upload(c, c->ev_begin, &c->d_ev_begin) ||
+        upload(c, c->ev_parts, &c->d_ev_parts) || upload(c, c->ev_pbegin, &c->d_ev_pbegin) ||
         upload(c, c->ev_lo, &c->d_ev_lo) || upload(c, c->ev_hi, &c->d_ev_hi))
       return MG_ERR_CUDA;
-    CK(cudaMalloc(&c->d_ev_out, std::max<size_t>(1, c->ev_items.size()) * 66 * sizeof(double)));
+    CK(cudaMalloc(&c->d_ev_out, (c->ev_parts.size() * kEvalPart + c->ev_items.size() * kEvalSeg + 1) * sizeof(double)));
     c->small_allocs.push_back(c->d_ev_out);
   }
   // ---- audio ----
@@ -3032,8 +3046,9 @@ mg_status mg_get_present(const mg_console* c, uint8_t* h_present) {
 
 mg_status mg_evaluate(mg_console* c, float* d_out) {
   if (!c || !d_out) return fail(c, MG_ERR_INVALID, "null pointer");
-  launch_eval(c->stream, c->d_songs, (int)c->songs.size(), c->d_ev_items, (int)c->ev_items.size(), c->d_ev_begin,
-              c->ev_seg_len, c->d_ev_lo, c->d_ev_hi, c->d_ev_out, d_out, c->tab.ptw);
+  launch_eval(c->stream, c->d_songs, (int)c->songs.size(), c->d_ev_parts, (int)c->ev_parts.size(), c->d_ev_items,
+              (int)c->ev_items.size(), c->d_ev_pbegin, c->d_ev_begin, c->ev_seg_len, c->d_ev_lo, c->d_ev_hi, c->d_ev_out,
+              c->d_ev_out + c->ev_parts.size() * kEvalPart, d_out, c->tab.ptw);
   CK(cudaGetLastError());
   return MG_OK;
 }

@@ -36,6 +36,8 @@ constexpr int kLossFrameBuf = 8192 + 512 + 128;   // padded frames of one loss w
 // floats of the loss adjoint's band gradients that fit next to the frames in the 227 KB of shared memory a
 // CTA may hold (1 KB left for the kernel's static shared memory)
 constexpr int kLossMaxDy = (227 * 1024 - 1024 - kLossFrameBuf * 8) / 4;
+constexpr int kEvalPiece = 16384;          // samples per evaluation piece (two Bark frames), two work items each
+constexpr int kEvalPart = 40, kEvalSeg = 8;  // doubles per evaluation work item / per segment
 constexpr int kEqOsM = 8192;               // overlap-save FFT size of the equalizer
 constexpr int kEqOsFwdBlock = kEqOsM - 2 * kEqHalf;        // 6146 outputs per forward block
 constexpr int kEqChunk = 8;                 // equalizer backward: blocks per work item (spectra summed in registers)
@@ -193,9 +195,9 @@ void launch_row_fwd_hz(const LaunchCtx&, const Item* items, int n, int maxN1);
 void launch_row_conv_fwd(const LaunchCtx&, const Item* items, int n, int maxN1, bool bwd_keep_u);
 void launch_col_inv_out(const LaunchCtx&, const Item* items, int n, int maxN2G);
 void launch_col_dybar(const LaunchCtx&, const Item* items, int n, int maxN2G);
-void launch_eval(cudaStream_t st, const SongDev* songs, int n_songs, const int2* items, int n_items,
-                 const int* item_begin, int seg_len, const int* band_lo, const int* band_hi, double* seg_out,
-                 float* out_song, const float2* ptw);
+void launch_eval(cudaStream_t st, const SongDev* songs, int n_songs, const int4* parts, int n_parts, const int2* segs,
+                 int n_segs, const int* seg_begin, const int* item_begin, int seg_len, const int* band_lo,
+                 const int* band_hi, double* part_out, double* seg_out, float* out_song, const float2* ptw);
 void init_eval_attributes();
 void launch_col_inv_out_keep(const LaunchCtx&, const Item* items, int n, int maxN2G);
 void launch_col_dybar_keep(const LaunchCtx&, const Item* items, int n, int maxN2G);
