@@ -247,12 +247,27 @@ __global__ void __launch_bounds__(256) k_chan_scale(LaunchCtx c, const int* __re
              (const void*)x, P.L, P.ld, (const void*)P.taps, (const void*)P.stats);
     return;
   }
+  // the samples of a thread are added in order, kScaleBatch of them loaded together (the strided loads are latency:
+  // 15.3 -> 13.8 us per launch on 16 nodes of 10 s)
+  constexpr int kScaleBatch = 4;
   const int nq = P.L >> 2;                    // whole quads of samples
-  for (int q = threadIdx.x * 32; q < nq; q += blockDim.x * 32) {   // every 32nd quad
-    const float4 a = reinterpret_cast<const float4*>(x)[q];
-    const float4 b = reinterpret_cast<const float4*>(x + P.ld)[q];
-    acc[0] += a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w;
-    acc[1] += b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w;
+  const float4* xl = reinterpret_cast<const float4*>(x);
+  const float4* xr = reinterpret_cast<const float4*>(x + P.ld);
+  const int qs = blockDim.x * 32;             // every 32nd quad
+  for (int q0 = threadIdx.x * 32; q0 < nq; q0 += kScaleBatch * qs) {
+    float4 a[kScaleBatch], b[kScaleBatch];
+#pragma unroll
+    for (int j = 0; j < kScaleBatch; ++j) {
+      const int q = min(q0 + j * qs, nq - 1);
+      a[j] = xl[q];
+      b[j] = xr[q];
+    }
+#pragma unroll
+    for (int j = 0; j < kScaleBatch; ++j)
+      if (q0 + j * qs < nq) {
+        acc[0] += a[j].x * a[j].x + a[j].y * a[j].y + a[j].z * a[j].z + a[j].w * a[j].w;
+        acc[1] += b[j].x * b[j].x + b[j].y * b[j].y + b[j].z * b[j].z + b[j].w * b[j].w;
+      }
   }
   if (which == 0 && P.type == T_D) {
     for (int j = threadIdx.x; j < kDlyTaps * kDlyFir; j += blockDim.x) {   // c_m of both channels
@@ -260,12 +275,24 @@ __global__ void __launch_bounds__(256) k_chan_scale(LaunchCtx c, const int* __re
       acc[2] += a * a;
       acc[3] += b * b;
     }
-  } else if (which == 0)
-    for (int j = threadIdx.x * 32; j < P.Nh; j += blockDim.x * 32) {   // every 32nd tap
-      const float2 t = tap_at(P, (int64_t)j + P.n0 >= 0 ? (int64_t)j + P.n0 : fft_len(P) + j + P.n0, fft_len(P));
-      acc[2] += t.x * t.x;
-      acc[3] += t.y * t.y;
+  } else if (which == 0) {
+    const int64_t N = fft_len(P);
+    const int js = blockDim.x * 32;           // every 32nd tap
+    for (int j0 = threadIdx.x * 32; j0 < P.Nh; j0 += kScaleBatch * js) {
+      float2 t[kScaleBatch];
+#pragma unroll
+      for (int k = 0; k < kScaleBatch; ++k) {
+        const int j = min(j0 + k * js, P.Nh - 1);
+        t[k] = tap_at(P, (int64_t)j + P.n0 >= 0 ? (int64_t)j + P.n0 : N + j + P.n0, N);
+      }
+#pragma unroll
+      for (int k = 0; k < kScaleBatch; ++k)
+        if (j0 + k * js < P.Nh) {
+          acc[2] += t[k].x * t[k].x;
+          acc[3] += t[k].y * t[k].y;
+        }
     }
+  }
   float out[4];
   block_sum<4>(acc, red, out);
   if (threadIdx.x == 0) {

@@ -178,7 +178,8 @@ __global__ void __launch_bounds__(kOsThreads) k_eq_dh_reduce(LaunchCtx c, const 
   const ProcDev& P = c.procs[procs[blockIdx.x]];
   for (int k = threadIdx.x; k < kOsM; k += blockDim.x) {
     float2 s = make_float2(0.f, 0.f);
-    for (int b = 0; b < P.nbpart; ++b) s = cadd(s, P.dhspec[(size_t)b * kOsM + k]);
+#pragma unroll 8
+    for (int b = 0; b < P.nbpart; ++b) s = cadd(s, P.dhspec[(size_t)b * kOsM + k]);   // in order, eight loads in flight
     sm[pidx(k)] = s;
   }
   __syncthreads();

@@ -16,28 +16,34 @@ __device__ __forceinline__ float softplusf_(float x) { return x > 20.f ? x : log
 // ------------------------------------------------------------------------------------------------
 // equalizer
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_eq_fir(LaunchCtx c, const int* __restrict__ procs) {
+// Both sums are serial chains of 1,023 dependent multiply-adds whose indices walk a 2,047-entry cosine table, so what
+// bounds them is latency: kEqParts CTAs per node, one output per thread (the taps at +n and -n share a sum).  With one
+// CTA per node and eight, resp. four, outputs per thread in turn they took 121 and 66 us per launch for any batch up to
+// a node per SM; now 22 and 23.
+constexpr int kEqParts = 8, kEqFirThreads = kEqParams / kEqParts;
+__global__ void __launch_bounds__(kEqFirThreads) k_eq_fir(LaunchCtx c, const int* __restrict__ procs) {
   __shared__ float ep[kEqParams];
   __shared__ float cs[kEqTaps];
   const ProcDev& P = c.procs[procs[blockIdx.x]];
   for (int k = threadIdx.x; k < kEqParams; k += blockDim.x) ep[k] = expf(P.p[k]);
   for (int m = threadIdx.x; m < kEqTaps; m += blockDim.x) cs[m] = c.tab.cos_eq[m];
   __syncthreads();
-  for (int j = threadIdx.x; j < kEqTaps; j += blockDim.x) {
-    const int an = abs(j - kEqHalf);
-    float acc = 0.f;
-    int idx = 0;
-    for (int k = 1; k < kEqParams; ++k) {
-      idx += an;
-      if (idx >= kEqTaps) idx -= kEqTaps;
-      acc = fmaf(ep[k], cs[idx], acc);
-    }
-    P.taps[j] = c.tab.hann_eq[j] * (ep[0] + 2.f * acc) * (1.f / kEqTaps);
+  const int an = blockIdx.y * kEqFirThreads + threadIdx.x;   // |n|
+  float acc = 0.f;
+  int idx = 0;
+#pragma unroll 8
+  for (int k = 1; k < kEqParams; ++k) {
+    idx += an;
+    if (idx >= kEqTaps) idx -= kEqTaps;
+    acc = fmaf(ep[k], cs[idx], acc);
   }
+  const int jp = kEqHalf + an, jm = kEqHalf - an;
+  P.taps[jp] = c.tab.hann_eq[jp] * (ep[0] + 2.f * acc) * (1.f / kEqTaps);
+  P.taps[jm] = c.tab.hann_eq[jm] * (ep[0] + 2.f * acc) * (1.f / kEqTaps);
 }
 
 // dL/dp_k = e^{p_k} (c_k / N) sum_n dh[n] v[n] cos(2 pi k n / N), c_0 = 1, c_k = 2; dh = dh_l + dh_r.
-__global__ void __launch_bounds__(256) k_eq_fir_adj(LaunchCtx c, const int* __restrict__ procs) {
+__global__ void __launch_bounds__(kEqFirThreads) k_eq_fir_adj(LaunchCtx c, const int* __restrict__ procs) {
   __shared__ float e[kEqParams];
   __shared__ float cs[kEqTaps];
   const ProcDev& P = c.procs[procs[blockIdx.x]];
@@ -49,16 +55,16 @@ __global__ void __launch_bounds__(256) k_eq_fir_adj(LaunchCtx c, const int* __re
     e[m] = m == 0 ? dp : dp + dm;
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < kEqParams; k += blockDim.x) {
-    float acc = e[0];
-    int idx = 0;
-    for (int m = 1; m <= kEqHalf; ++m) {
-      idx += k;
-      if (idx >= kEqTaps) idx -= kEqTaps;
-      acc = fmaf(e[m], cs[idx], acc);
-    }
-    P.gp[k] = expf(P.p[k]) * (k == 0 ? 1.f : 2.f) * (1.f / kEqTaps) * acc;
+  const int k = blockIdx.y * kEqFirThreads + threadIdx.x;
+  float acc = e[0];
+  int idx = 0;
+#pragma unroll 8
+  for (int m = 1; m <= kEqHalf; ++m) {
+    idx += k;
+    if (idx >= kEqTaps) idx -= kEqTaps;
+    acc = fmaf(e[m], cs[idx], acc);
   }
+  P.gp[k] = expf(P.p[k]) * (k == 0 ? 1.f : 2.f) * (1.f / kEqTaps) * acc;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -474,19 +480,24 @@ __global__ void __launch_bounds__(512) k_rev_adj(LaunchCtx c, const Item* __rest
   }
 }
 
-__global__ void __launch_bounds__(256) k_rev_adj_fin(LaunchCtx c, const int* __restrict__ procs) {
+// One thread per bin; the frame groups' partials are added in order, eight loads in flight (one at a time: 23 us).
+__global__ void __launch_bounds__(2 * kRevParams) k_rev_adj_fin(LaunchCtx c, const int* __restrict__ procs) {
   const ProcDev& P = c.procs[procs[blockIdx.x]];
   const int ng = (P.nframes + kRevFG - 1) / kRevFG;
   for (int e = threadIdx.x; e < 2 * kRevParams; e += blockDim.x) {
     const int x = e / kRevParams, k = e % kRevParams;
     float a0 = 0.f, a1 = 0.f;
+    const float2* part = reinterpret_cast<const float2*>(P.aux) + (size_t)x * ng * kRevBins + k;
+    const bool nyq = k == kRevParams - 1;   // the Nyquist bin reuses parameter 191
+#pragma unroll 8
     for (int g = 0; g < ng; ++g) {
-      const float* part = P.aux + ((size_t)x * ng + g) * kRevBins * 2;
-      a0 += part[k * 2];
-      a1 += part[k * 2 + 1];
-      if (k == kRevParams - 1) {   // the Nyquist bin reuses parameter 191
-        a0 += part[(kRevBins - 1) * 2];
-        a1 += part[(kRevBins - 1) * 2 + 1];
+      const float2 v = part[(size_t)g * kRevBins];
+      a0 += v.x;
+      a1 += v.y;
+      if (nyq) {
+        const float2 w = part[(size_t)g * kRevBins + 1];
+        a0 += w.x;
+        a1 += w.y;
       }
     }
     P.gp[x * 2 * kRevParams + k] = a0;
@@ -495,10 +506,10 @@ __global__ void __launch_bounds__(256) k_rev_adj_fin(LaunchCtx c, const int* __r
 }
 
 void launch_eq_fir(const LaunchCtx& c, const int* procs, int n) {
-  if (n) k_eq_fir<<<n, 256, 0, c.stream>>>(c, procs);
+  if (n) k_eq_fir<<<dim3(n, kEqParts), kEqFirThreads, 0, c.stream>>>(c, procs);
 }
 void launch_eq_fir_adj(const LaunchCtx& c, const int* procs, int n) {
-  if (n) k_eq_fir_adj<<<n, 256, 0, c.stream>>>(c, procs);
+  if (n) k_eq_fir_adj<<<dim3(n, kEqParts), kEqFirThreads, 0, c.stream>>>(c, procs);
 }
 void launch_dly_prep(const LaunchCtx& c, const int* procs, int n) {
   if (n) k_dly_prep<<<n, 256, 0, c.stream>>>(c, procs);
@@ -521,7 +532,7 @@ void init_fir_attributes() {
   cudaFuncSetAttribute(k_rev_noise_stft, cudaFuncAttributeMaxDynamicSharedMemorySize, kRevFG * kRevFft * (int)sizeof(float2));
 }
 void launch_rev_adj_fin(const LaunchCtx& c, const int* procs, int n) {
-  if (n) k_rev_adj_fin<<<n, 256, 0, c.stream>>>(c, procs);
+  if (n) k_rev_adj_fin<<<n, 2 * kRevParams, 0, c.stream>>>(c, procs);
 }
 void launch_rev_noise_stft(const LaunchCtx& c, const Item* items, int n, const float* noise, int noise_len) {
   if (n) k_rev_noise_stft<<<n, 512, kRevFG * kRevFft * sizeof(float2), c.stream>>>(c, items, noise, noise_len);
