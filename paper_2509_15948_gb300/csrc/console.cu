@@ -216,7 +216,7 @@ struct mg_console {
   int n_msum = 0;
   ProcList all_present;
   ProcList all_lti_present;
-  DevVec<int4> loss_items[3];
+  DevVec<int4> loss_items;       // of every resolution, song-major
   ItemList gather_items;
   // evaluation metrics (Sec. 5.3): (song, 8 s segment) items, per-song item ranges, the work items of every segment's
   // pieces (song, segment, 2 piece + signal) with per-segment ranges, Bark band bin ranges
@@ -253,8 +253,8 @@ struct mg_console {
   int cur_stage = 9;
   double stage_ms[10] = {0};
   int64_t stage_n[10] = {0};
-  // loss items of one song (per resolution: first item, count) for per-song target refresh
-  std::vector<std::array<int2, 3>> song_litems;
+  // loss items of one song (first item, count) for per-song target refresh
+  std::vector<int2> song_litems;
   bool capturing = false;
   std::vector<void*> small_allocs;
 };
@@ -809,13 +809,11 @@ void render(mg_console* c, const LaunchCtx& x) {
 
 void loss_forward(mg_console* c, const LaunchCtx& x, int mode, float* out_losses, float* out_la, int la_stride) {
   StageScope scope(c, 7);
-  for (int r = 0; r < c->nres; ++r) {
-    auto& L = c->loss_items[r];
-    if (!L.h.empty())
-      run(c, F_LOSS_FWD, [&] {   // frame kernel: 0 target spectrogram, 1 loss partials (losses and trials)
-        launch_loss_frames(x, c->d_songs, c->d_res, L.d, (int)L.h.size(), mode == 0 ? 0 : (mode == 1 ? 3 : 1), c->loss_max_dy);
-      });
-  }
+  auto& L = c->loss_items;
+  if (!L.h.empty())
+    run(c, F_LOSS_FWD, [&] {   // frame kernel: 0 target spectrogram, 1 loss partials (losses and trials)
+      launch_loss_frames(x, c->d_songs, c->d_res, L.d, (int)L.h.size(), mode == 0 ? 0 : (mode == 1 ? 3 : 1), c->loss_max_dy);
+    });
   if (mode != 0) run_procs(c, F_FINALIZE, c->all_lti_present, [&](const int* p, int n) { launch_node_stats(x, p, n, 1); });
   run(c, F_FINALIZE, [&] {
     launch_loss_finalize_mode(x, c->d_songs, (int)c->songs.size(), c->d_res, c->nres, c->d_alphas, mode, out_losses,
@@ -826,11 +824,9 @@ void loss_forward(mg_console* c, const LaunchCtx& x, int mode, float* out_losses
 void backward_pass(mg_console* c, const LaunchCtx& x) {
   {
     StageScope scope(c, 7);
-    for (int r = 0; r < c->nres; ++r) {
-      auto& L = c->loss_items[r];
-      if (!L.h.empty())
-        run(c, F_LOSS_BWD, [&] { launch_loss_frames(x, c->d_songs, c->d_res, L.d, (int)L.h.size(), 2, c->loss_max_dy); });
-    }
+    auto& L = c->loss_items;
+    if (!L.h.empty())
+      run(c, F_LOSS_BWD, [&] { launch_loss_frames(x, c->d_songs, c->d_res, L.d, (int)L.h.size(), 2, c->loss_max_dy); });
     run_items(c, F_LOSS_GATHER, c->gather_items,
               [&](const Item* it, int n) { launch_loss_gather(x, c->d_songs, c->d_res, c->nres, it, n); });
   }
@@ -1554,26 +1550,27 @@ mg_status autotune_splits(mg_console* c) {
   return MG_OK;
 }
 
-// Loss work items for the current frames per item (song-major within each resolution, so one song's items are
-// one contiguous range), with the per-song item counts and the resolutions' item length on the device.
+// Loss work items for the current frames per item, one list over all resolutions (song-major, so one song's items are
+// one contiguous range; a launch per resolution was a wave or two of CTAs each), with the per-song item counts and
+// the resolutions' item length on the device.
 mg_status build_loss_items(mg_console* c) {
-  c->song_litems.assign(c->songs.size(), std::array<int2, 3>{});
-  for (int r = 0; r < c->nres; ++r) {
-    auto& L = c->loss_items[r];
-    L.h.clear();
-    const int per = c->loss_per[r];
-    c->hres[r].per = per;
-    for (size_t si = 0; si < c->songs.size(); ++si) {
-      HostSong& hs = c->songs[si];
-      const int first = (int)L.h.size();
+  c->song_litems.assign(c->songs.size(), int2{0, 0});
+  auto& L = c->loss_items;
+  L.h.clear();
+  for (int r = 0; r < c->nres; ++r) c->hres[r].per = c->loss_per[r];
+  for (size_t si = 0; si < c->songs.size(); ++si) {
+    HostSong& hs = c->songs[si];
+    const int first = (int)L.h.size();
+    for (int r = 0; r < c->nres; ++r) {
+      const int per = c->loss_per[r], begin = (int)L.h.size();
       for (int t = hs.first[r]; t < hs.nframes[r]; t += per)
         L.h.push_back(make_int4((int)si, r, t, std::min(per, hs.nframes[r] - t)));
-      c->song_litems[si][r] = make_int2(first, (int)L.h.size() - first);
-      hs.litems[r] = (int)L.h.size() - first;
+      hs.litems[r] = (int)L.h.size() - begin;
       c->hsd[si].litems[r] = hs.litems[r];
     }
-    if (upload(c, L.h, &L.d) != MG_OK) return MG_ERR_CUDA;
+    c->song_litems[si] = make_int2(first, (int)L.h.size() - first);
   }
+  if (upload(c, L.h, &L.d) != MG_OK) return MG_ERR_CUDA;
   if (upload(c, c->hsd, &c->d_songs) != MG_OK || upload(c, c->hres, &c->d_res) != MG_OK) return MG_ERR_CUDA;
   return MG_OK;
 }
@@ -1647,12 +1644,9 @@ mg_status autotune_packing(mg_console* c) {
     if (set_div(div) != MG_OK) return MG_ERR_CUDA;
     LaunchCtx x = make_ctx(c, nullptr);
     auto pass = [&] {
-      for (int r = 0; r < c->nres; ++r) {
-        auto& L = c->loss_items[r];
-        if (L.h.empty()) continue;
-        launch_loss_frames(x, c->d_songs, c->d_res, L.d, (int)L.h.size(), 1, c->loss_max_dy);
-        launch_loss_frames(x, c->d_songs, c->d_res, L.d, (int)L.h.size(), 2, c->loss_max_dy);
-      }
+      auto& L = c->loss_items;
+      launch_loss_frames(x, c->d_songs, c->d_res, L.d, (int)L.h.size(), 1, c->loss_max_dy);
+      launch_loss_frames(x, c->d_songs, c->d_res, L.d, (int)L.h.size(), 2, c->loss_max_dy);
     };
     pass();
     float ms = 1e30f;
@@ -1898,7 +1892,7 @@ mg_status create_impl(mg_console* c, const mg_console_desc* d, const mg_song_des
   c->gather_items = ItemList{};
   for (size_t si = 0; si < c->songs.size(); ++si) {
     c->gather_items.beg.push_back((int)c->gather_items.h.size());
-    for (int t = 0; t < (c->songs[si].L + kElemTile - 1) / kElemTile; ++t) c->gather_items.h.push_back(Item{(int)si, t});
+    for (int t = 0; t < (c->songs[si].L + kGatherTile - 1) / kGatherTile; ++t) c->gather_items.h.push_back(Item{(int)si, t});
   }
   c->gather_items.beg.push_back((int)c->gather_items.h.size());
   if (upload_items(c, c->gather_items) != MG_OK) return MG_ERR_CUDA;
@@ -2090,7 +2084,7 @@ struct ScoreChunk {
   std::vector<int> sum_beg, sum_L, sum_ld;
   ItemList m_items, o_items;
   std::vector<SongDev> vs;
-  std::vector<int4> litems[3];
+  std::vector<int4> litems;
   std::vector<int> map;                      // [candidate][song]: song copy, or -1 (unchanged)
   std::vector<std::vector<std::pair<char*, const char*>>> promo;   // [candidate][song]: (arena, copy) buffers
   size_t table_begin = 0;                    // workspace offset of the tables (copied from the host blob)
@@ -2106,7 +2100,7 @@ struct ScoreChunk {
   ProcDev* d_vp = nullptr;
   uint8_t* d_vmask = nullptr;
   SongDev* d_vs = nullptr;
-  int4* d_litems[3] = {nullptr, nullptr, nullptr};
+  int4* d_litems = nullptr;
   float** d_sum_out = nullptr;
   const float** d_sum_in = nullptr;
   int *d_sum_beg = nullptr, *d_sum_L = nullptr, *d_sum_ld = nullptr;
@@ -2352,7 +2346,7 @@ void build_chunk(mg_console* c, const std::vector<CandPlan>& plans, const uint8_
       for (int r = 0; r < c->nres; ++r) {
         const int per = c->loss_per[r];
         for (int t = hs.first[r]; t < hs.nframes[r]; t += per)
-          k.litems[r].push_back(make_int4(vsi, r, t, std::min(per, hs.nframes[r] - t)));
+          k.litems.push_back(make_int4(vsi, r, t, std::min(per, hs.nframes[r] - t)));
       }
       k.map[(size_t)(j - j0) * ns + si] = vsi;
       k.promo[(size_t)(j - j0) * ns + si].push_back({A(hs.o_mix), (const char*)mix});
@@ -2426,7 +2420,7 @@ void build_chunk(mg_console* c, const std::vector<CandPlan>& plans, const uint8_
   k.d_vmask = w.table(k.vmask);
   k.d_map = w.table(k.map);
   k.d_vs = w.table(k.vs);
-  for (int r = 0; r < 3; ++r) k.d_litems[r] = w.table(k.litems[r]);
+  k.d_litems = w.table(k.litems);
   k.d_sum_out = w.table(k.sum_out);
   k.d_sum_in = w.table(k.sum_in);
   k.d_sum_beg = w.table(k.sum_beg);
@@ -2508,9 +2502,8 @@ std::string check_chunk(const mg_console* c, const ScoreChunk& k) {
   for (const SongDev& sd : k.vs)
     if (!in(sd.mix, (size_t)2 * sd.ld * sizeof(float)) || !in(sd.lpart, (size_t)18 * sd.lcap * sizeof(float)))
       return "song copy buffers out of range";
-  for (int r = 0; r < 3; ++r)
-    for (const int4& it : k.litems[r])
-      if (it.x < 0 || it.x >= (int)k.vs.size()) return "loss item indexes a missing song copy";
+  for (const int4& it : k.litems)
+    if (it.x < 0 || it.x >= (int)k.vs.size()) return "loss item indexes a missing song copy";
   return std::string();
 }
 
@@ -2674,11 +2667,10 @@ mg_status prune_scores_batched(mg_console* c, const uint8_t* d_masks, int n_mask
         });
       }
       StageScope scope(c, 7);
-      for (int r = 0; r < c->nres; ++r)
-        if (!k.litems[r].empty())
-          run(c, F_LOSS_FWD, [&] {
-            launch_loss_frames(xv, k.d_vs, c->d_res, k.d_litems[r], (int)k.litems[r].size(), 1, c->loss_max_dy);
-          });
+      if (!k.litems.empty())
+        run(c, F_LOSS_FWD, [&] {
+          launch_loss_frames(xv, k.d_vs, c->d_res, k.d_litems, (int)k.litems.size(), 1, c->loss_max_dy);
+        });
       run(c, F_FINALIZE, [&] {
         launch_loss_finalize_mode(xv, k.d_vs, (int)k.vs.size(), c->d_res, c->nres, c->d_alphas, 2, nullptr, k.vla, 1);
       });
@@ -3082,10 +3074,8 @@ mg_status mg_update_audio(mg_console* c, int32_t song, const float* sources, con
                          (size_t)hs.L * sizeof(float), 2, k, c->stream));
     // target spectrograms and their norms of this song only
     LaunchCtx x = make_ctx(c, nullptr);
-    for (int r = 0; r < c->nres; ++r) {
-      const int2 rg = c->song_litems[song][r];
-      if (rg.y > 0) launch_loss_frames(x, c->d_songs, c->d_res, c->loss_items[r].d + rg.x, rg.y, 0, c->loss_max_dy);
-    }
+    const int2 rg = c->song_litems[song];
+    if (rg.y > 0) launch_loss_frames(x, c->d_songs, c->d_res, c->loss_items.d + rg.x, rg.y, 0, c->loss_max_dy);
     launch_loss_finalize_mode(x, c->d_songs + song, 1, c->d_res, c->nres, c->d_alphas, 0, nullptr, nullptr, 0);
   }
   c->fwd_valid = false;

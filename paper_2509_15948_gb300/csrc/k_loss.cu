@@ -8,6 +8,13 @@
 // Adjoint: the same frames are re-transformed, dL/dY_hat per band goes back to the bins through the
 // transposed Mel CSR, to the complex bins through |X|, to the packed Hermitian spectrum, and through one
 // inverse FFT to the windowed frame; a gather kernel overlap-adds the frames of all resolutions.
+//
+// What bounds it: with two CTAs per SM (64 registers, 69-94 KB) a work item is latency.  The Mel sums and the adjoint's
+// band values went one (frame, band) after the other, each waiting for its own table and target loads and for 20
+// shuffles, 45 us per wave of CTAs whatever the resolution.  Four values of a thread or warp now go together with
+// the target loaded before the sums, the warp sums take 7 shuffles, the four channels of a bin share its weights,
+// and all resolutions are one launch.  On one 30 s mix forward, adjoint and overlap-add took 780 us, now 270.
+// Every sum keeps its order, so the losses and gradients keep their bits.
 #include "mg_fftp.cuh"
 
 namespace mg {
@@ -62,9 +69,10 @@ __device__ __forceinline__ float4 bin_mags(const LossRes& R, const float2* Z, in
 // mode 1: partial sums of |dlog| and (Y - Yhat)^2 per set; mode 3: mode 1 that also keeps the frame spectra
 // (in dF, which the adjoint overwrites frame by frame) and the band values Yhat (training forward);
 // mode 2: adjoint frames to dF from the kept spectra and band values.
+template <int mode>
 __global__ void __launch_bounds__(kLossThreads, 2) k_loss_frames(LaunchCtx c, const SongDev* __restrict__ songs,
                                                               const LossRes* __restrict__ resv,
-                                                              const int4* __restrict__ items, int mode) {
+                                                              const int4* __restrict__ items) {
   extern __shared__ float2 sm[];
   __shared__ float red[6 * 32];
   const int4 it = items[blockIdx.x];
@@ -73,12 +81,15 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_loss_frames(LaunchCtx c, co
   const int t0 = it.z, nb = it.w, n = R.nfft, nbands = R.nbands, bs = pstride(n);
   const float* x = mode == 0 ? S.target : S.mix;
   float2* Zk = reinterpret_cast<float2*>(S.dF[it.y]);     // frame spectra kept between mode 3 and mode 2
-  if (mode == 2) {
-    for (int e = threadIdx.x; e < nb * n; e += blockDim.x) {
-      const int f = e >> R.log_nfft, j = e & (n - 1);
-      sm[f * bs + pidx(j)] = Zk[(size_t)(t0 + f) * n + j];
+  if constexpr (mode == 2) {
+    const float4* zi = reinterpret_cast<const float4*>(Zk + (size_t)t0 * n);
+#pragma unroll 4
+    for (int e = threadIdx.x; e < nb * n / 2; e += blockDim.x) {
+      const int f = e >> (R.log_nfft - 1), j = 2 * e & (n - 1);
+      const float4 z = zi[e];
+      sm[f * bs + pidx(j)] = make_float2(z.x, z.y);
+      sm[f * bs + pidx(j + 1)] = make_float2(z.z, z.w);
     }
-    __syncthreads();
   } else {
     // the windowed frames go straight from global memory into the first pass of the transform
     const int L = S.L, ld = S.ld, hop = R.hop;
@@ -88,22 +99,23 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_loss_frames(LaunchCtx c, co
       const float w = win[j];
       return s < L ? make_float2(x[s] * w, x[ld + s] * w) : make_float2(0.f, 0.f);
     });
-    if (mode == 3)
-      for (int e = threadIdx.x; e < nb * n; e += blockDim.x) {
-        const int f = e >> R.log_nfft, j = e & (n - 1);
-        Zk[(size_t)(t0 + f) * n + j] = sm[f * bs + pidx(j)];
-      }
   }
   float* Yt = S.Y[it.y];
   float* Yk = S.Yh[it.y];
-  if (mode != 2) {
+  if constexpr (mode != 2) {
     // magnitudes of the four channels per bin, in place (each thread owns the pair k, n - k; the thread of
-    // k = 0 also takes k = n/2)
+    // k = 0 also takes k = n/2); mode 3 keeps the spectrum on the way
     const int half = n >> 1, lh = R.log_nfft - 1;
-    __syncthreads();   // mode 3: every thread has copied its part of the spectrum out
+#pragma unroll 2
     for (int e = threadIdx.x; e < nb << lh; e += blockDim.x) {
       const int f = e >> lh, k = e & (half - 1);
       float2* Z = sm + f * bs;
+      if (mode == 3) {
+        float2* zo = Zk + (size_t)(t0 + f) * n;
+        const int k2 = k == 0 ? half : n - k;
+        zo[k] = Z[pidx(k)];
+        zo[k2] = Z[pidx(k2)];
+      }
       if (k == 0) {
         const float4 m0 = bin_mags(R, Z, 0), mh = bin_mags(R, Z, half);
         Z[pidx(0)] = make_float2(m0.x, m0.y);
@@ -121,55 +133,142 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_loss_frames(LaunchCtx c, co
     // (frame, band, channel); with wide ones one warp per (frame, band), its lanes striding the band's bins and
     // the four channel sums reduced over the warp (a fixed xor order), so a wide high band no longer holds the
     // whole block at the barrier behind one thread
-    float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    auto band_out = [&](int f, int b, int ch, float yh) {
-      const int set = ch < 2 ? 0 : ch - 1;
-      const size_t yi = ((size_t)(t0 + f) * nbands + b) * 4 + ch;
-      float* ydst = Yt + yi;
-      if (mode == 3) Yk[yi] = yh;
-      if (mode == 0) {
-        *ydst = yh;
-        acc[set] += yh * yh;
-      } else {
-        const float y = *ydst;
-        acc[2 * set] += fabsf(logf(y + kLogEps) - logf(yh + kLogEps));
-        const float d = y - yh;
-        acc[2 * set + 1] += d * d;
-      }
-    };
+    // a thread only ever adds terms of one channel, so two scalars hold its sums
+    float acc0 = 0.f, acc1 = 0.f;
+    int mych = threadIdx.x & 3;
     if (R.band_beg[nbands] >= 16 * nbands) {
-      const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-      for (int e = wid; e < nb * nbands; e += nw) {
-        const int f = e / nbands, b = e - f * nbands;
-        const float2* Zf = sm + f * bs;
-        float y4[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int q = R.band_beg[b] + lane; q < R.band_beg[b + 1]; q += 32) {
-          const int k = R.band_bin[q];
-          const float wq = R.band_w[q];
-          const float2 lr = Zf[pidx(k)], ms = Zf[mag_slot2(k, n)];
-          y4[0] = fmaf(wq, lr.x, y4[0]);
-          y4[1] = fmaf(wq, lr.y, y4[1]);
-          y4[2] = fmaf(wq, ms.x, y4[2]);
-          y4[3] = fmaf(wq, ms.y, y4[3]);
+      // a warp takes kWide (frame, band) pairs together, so that their loads and shuffles overlap; after the sums lane
+      // l finishes pair l & 7 of channel chan_of(l), and lanes 0..3 add the pairs' loss terms in pair order
+      const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5, total = nb * nbands;
+      constexpr int kWide = 4;
+      const int lch = ((lane >> 4) & 1) * 2 + ((lane >> 3) & 1);
+      for (int e0 = wid; e0 < total; e0 += kWide * nw) {
+        float y4[kWide][4];
+        int beg[kWide], len[kWide], most = 0;
+        const float2* Zf[kWide];
+#pragma unroll
+        for (int j = 0; j < kWide; ++j) {
+          const int e = e0 + j * nw, ee = e < total ? e : e0;
+          const int f = ee / nbands, b = ee - f * nbands;
+          Zf[j] = sm + f * bs;
+          beg[j] = R.band_beg[b];
+          len[j] = e < total ? R.band_beg[b + 1] - beg[j] : 0;
+          most = max(most, len[j]);
+#pragma unroll
+          for (int c4 = 0; c4 < 4; ++c4) y4[j][c4] = 0.f;
         }
+        // this lane's pair and channel: its target (or earlier) value is on its way during the sums
+        const int em = e0 + (lane & 7) * nw;
+        const bool mine = (lane & 7) < kWide && em < total;
+        const size_t yi = mine ? ((size_t)t0 * nbands + em) * 4 + lch : 0;
+        const float yt = mine && mode != 0 ? Yt[yi] : 0.f;
+        for (int q = lane; q < most; q += 32) {
 #pragma unroll
-        for (int c4 = 0; c4 < 4; ++c4)
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) y4[c4] += __shfl_xor_sync(0xffffffffu, y4[c4], o);
-        if (lane < 4) band_out(f, b, lane, lane == 0 ? y4[0] : lane == 1 ? y4[1] : lane == 2 ? y4[2] : y4[3]);
-      }
-    } else {
-      for (int e = threadIdx.x; e < nb * nbands * 4; e += blockDim.x) {
-        const int f = e / (nbands * 4), r = e - f * (nbands * 4), b = r >> 2, ch = r & 3;
-        const float* Zf = reinterpret_cast<const float*>(sm + f * bs);
+          for (int j = 0; j < kWide; ++j) {
+            if (q < len[j]) {
+              const int k = R.band_bin[beg[j] + q];
+              const float wq = R.band_w[beg[j] + q];
+              const float2 lr = Zf[j][pidx(k)], ms = Zf[j][mag_slot2(k, n)];
+              y4[j][0] = fmaf(wq, lr.x, y4[j][0]);
+              y4[j][1] = fmaf(wq, lr.y, y4[j][1]);
+              y4[j][2] = fmaf(wq, ms.x, y4[j][2]);
+              y4[j][3] = fmaf(wq, ms.y, y4[j][3]);
+            }
+          }
+        }
+        // warp sums over xor 16, 8, 4, 2, 1 (in that order for every channel): after the first step a lane keeps two
+        // channels, after the second one
         float yh = 0.f;
-        for (int q = R.band_beg[b]; q < R.band_beg[b + 1]; ++q) {
-          const int k = R.band_bin[q];
-          const int slot = ch < 2 ? pidx(k) : mag_slot2(k, n);
-          yh = fmaf(R.band_w[q], Zf[2 * slot + (ch & 1)], yh);
+#pragma unroll
+        for (int j = 0; j < kWide; ++j) {
+          const bool h16 = lane & 16, h8 = lane & 8;
+          const float s0 = __shfl_xor_sync(0xffffffffu, h16 ? y4[j][0] : y4[j][2], 16);
+          const float s1 = __shfl_xor_sync(0xffffffffu, h16 ? y4[j][1] : y4[j][3], 16);
+          const float a0 = (h16 ? y4[j][2] : y4[j][0]) + s0, a1 = (h16 ? y4[j][3] : y4[j][1]) + s1;
+          float v = (h8 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, h8 ? a0 : a1, 8);
+          v += __shfl_xor_sync(0xffffffffu, v, 4);
+          v += __shfl_xor_sync(0xffffffffu, v, 2);
+          v += __shfl_xor_sync(0xffffffffu, v, 1);
+          if ((lane & 7) == j) yh = v;
         }
-        band_out(f, b, ch, yh);
+        float d0 = 0.f, d1 = 0.f;
+        if (mine) {
+          if (mode == 3) Yk[yi] = yh;
+          if (mode == 0) {
+            Yt[yi] = yh;
+          } else {
+            d0 = fabsf(logf(yt + kLogEps) - logf(yh + kLogEps));
+            d1 = yt - yh;
+          }
+        }
+        // lane c < 4 adds channel c of the pairs in order; the lane of pair j, channel c is 16 (c / 2) + 8 (c mod 2) + j
+#pragma unroll
+        for (int j = 0; j < kWide; ++j) {
+          const int src = (lane & 2) * 8 + (lane & 1) * 8 + j;
+          const float x0 = __shfl_sync(0xffffffffu, d0, src), x1 = __shfl_sync(0xffffffffu, d1, src);
+          const float xh = __shfl_sync(0xffffffffu, yh, src);
+          if (lane < 4 && e0 + j * nw < total) {
+            if (mode == 0) {
+              acc0 += xh * xh;
+            } else {
+              acc0 += x0;
+              acc1 += x1 * x1;
+            }
+          }
+        }
       }
+      mych = lane & 3;   // lanes 0..3 hold the sums of channels 0..3, the others zeros
+    } else {
+      // a thread takes kNarrow (frame, band) values of its channel together (loads in flight)
+      constexpr int kNarrow = 4;
+      const int total = nb * nbands * 4, nth = blockDim.x, ch = mych;
+      for (int e0 = threadIdx.x; e0 < total; e0 += kNarrow * nth) {
+        const float* Zf[kNarrow];
+        float yh[kNarrow], yt[kNarrow];
+        int beg[kNarrow], len[kNarrow], most = 0;
+#pragma unroll
+        for (int j = 0; j < kNarrow; ++j) {
+          const int e = e0 + j * nth, ee = e < total ? e : e0;
+          const int f = ee / (nbands * 4), b = (ee - f * (nbands * 4)) >> 2;
+          Zf[j] = reinterpret_cast<const float*>(sm + f * bs);
+          yt[j] = e < total && mode != 0 ? Yt[(size_t)t0 * nbands * 4 + e] : 0.f;
+          beg[j] = R.band_beg[b];
+          len[j] = e < total ? R.band_beg[b + 1] - beg[j] : 0;
+          most = max(most, len[j]);
+          yh[j] = 0.f;
+        }
+        for (int q = 0; q < most; ++q) {
+#pragma unroll
+          for (int j = 0; j < kNarrow; ++j) {
+            if (q < len[j]) {
+              const int k = R.band_bin[beg[j] + q];
+              const int slot = ch < 2 ? pidx(k) : mag_slot2(k, n);
+              yh[j] = fmaf(R.band_w[beg[j] + q], Zf[j][2 * slot + (ch & 1)], yh[j]);
+            }
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < kNarrow; ++j) {
+          const int e = e0 + j * nth;
+          if (e >= total) continue;
+          const size_t yi = (size_t)t0 * nbands * 4 + e;
+          if (mode == 3) Yk[yi] = yh[j];
+          if (mode == 0) {
+            Yt[yi] = yh[j];
+            acc0 += yh[j] * yh[j];
+          } else {
+            acc0 += fabsf(logf(yt[j] + kLogEps) - logf(yh[j] + kLogEps));
+            const float d = yt[j] - yh[j];
+            acc1 += d * d;
+          }
+        }
+      }
+    }
+    float acc[6];
+    {
+      const int set = mych < 2 ? 0 : mych - 1;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) acc[k] = mode == 0 ? (k == set ? acc0 : 0.f) : (k == 2 * set ? acc0 : (k == 2 * set + 1 ? acc1 : 0.f));
     }
     float out[6];
     block_sum<6>(acc, red, out);
@@ -178,20 +277,22 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_loss_frames(LaunchCtx c, co
       const int row = (t0 - S.first_frame[it.y]) / R.per;
       for (int j = 0; j < 6; ++j) S.lpart[((size_t)it.y * S.lcap + row) * 6 + j] = out[j];
     }
-    return;
-  }
+  } else {
   // ---- adjoint ----
   float* dY = reinterpret_cast<float*>(sm + kFrameBuf);   // [nb][nbands][4]
   const float* coef = S.coef + it.y * 6;                    // per set: (alpha / count, alpha / (|Y - Yh| |Y|))
-  for (int e = threadIdx.x; e < nb * nbands * 4; e += blockDim.x) {
-    const int f = e / (nbands * 4), r = e % (nbands * 4), b = r >> 2, ch = r & 3;
-    const size_t yi = ((size_t)(t0 + f) * nbands + b) * 4 + ch;
-    const float yh = Yk[yi];
-    const int set = ch < 2 ? 0 : ch - 1;
-    const float y = Yt[yi];
-    const float dl = logf(yh + kLogEps) - logf(y + kLogEps);
-    const float sg = dl > 0.f ? 1.f : (dl < 0.f ? -1.f : 0.f);
-    dY[e] = coef[2 * set] * sg / (yh + kLogEps) + coef[2 * set + 1] * (yh - y);
+  {
+    // item-contiguous band values: entry e of the item is value e of its first frame's row
+    const float *yk = Yk + (size_t)t0 * nbands * 4, *yt = Yt + (size_t)t0 * nbands * 4;
+    const int ch = threadIdx.x & 3, set = ch < 2 ? 0 : ch - 1;
+    const float c0 = coef[2 * set], c1 = coef[2 * set + 1];
+#pragma unroll 4
+    for (int e = threadIdx.x; e < nb * nbands * 4; e += blockDim.x) {
+      const float yh = yk[e], y = yt[e];
+      const float dl = logf(yh + kLogEps) - logf(y + kLogEps);
+      const float sg = dl > 0.f ? 1.f : (dl < 0.f ? -1.f : 0.f);
+      dY[e] = c0 * sg / (yh + kLogEps) + c1 * (yh - y);
+    }
   }
   __syncthreads();
   // bins -> packed Hermitian spectrum, in place (thread owns the pair k, n - k)
@@ -203,13 +304,23 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_loss_frames(LaunchCtx c, co
     bin_spectra(Z, k, n, XL, XR);
     const float* dYf = dY + (size_t)f * nbands * 4;
     float2 gl = make_float2(0.f, 0.f), gr = gl;
+    float dmv[4] = {0.f, 0.f, 0.f, 0.f};
+    const int qe = R.bin_beg[k + 1];
+    for (int q = R.bin_beg[k]; q < qe; ++q) {   // the four channels of a band together
+      const float wq = R.bin_w[q];
+      const float4 d = reinterpret_cast<const float4*>(dYf)[R.bin_band[q]];
+      dmv[0] = fmaf(wq, d.x, dmv[0]);
+      dmv[1] = fmaf(wq, d.y, dmv[1]);
+      dmv[2] = fmaf(wq, d.z, dmv[2]);
+      dmv[3] = fmaf(wq, d.w, dmv[3]);
+    }
+    const float aw2 = R.aw2[k];
 #pragma unroll
     for (int ch = 0; ch < 4; ++ch) {
-      float dm = 0.f;
-      for (int q = R.bin_beg[k]; q < R.bin_beg[k + 1]; ++q) dm = fmaf(R.bin_w[q], dYf[R.bin_band[q] * 4 + ch], dm);
+      const float dm = dmv[ch];
       const float2 X = chan(ch, XL, XR);
-      const float mag = sqrtf(R.aw2[k] * (X.x * X.x + X.y * X.y) + kMagEps);
-      const float2 g = cscale(X, dm * R.aw2[k] / mag);
+      const float mag = sqrtf(aw2 * (X.x * X.x + X.y * X.y) + kMagEps);
+      const float2 g = cscale(X, dm * aw2 / mag);
       if (ch == 0) gl = cadd(gl, g);
       else if (ch == 1) gr = cadd(gr, g);
       else if (ch == 2) { gl = cadd(gl, g); gr = cadd(gr, g); }
@@ -229,6 +340,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_loss_frames(LaunchCtx c, co
   const float* win = R.win;
   fft_p_io<true>(sm, R.log_nfft, nb, bs, c.tab.ptw, fftp::SmemIO(),
                  [=](int f, int j, float2 v) { dF[(size_t)f * n + j] = cscale(v, win[j]); });
+  }
 }
 
 // dmix[c][s] = sum over resolutions and covering frames of dF (overlap-add, fixed order)
@@ -236,8 +348,8 @@ __global__ void __launch_bounds__(256) k_loss_gather(const SongDev* __restrict__
                                                     int nres, const Item* __restrict__ items) {
   const Item it = items[blockIdx.x];
   const SongDev& S = songs[it.proc];
-  const int s0 = it.idx * kElemTile;
-  for (int s = s0 + threadIdx.x; s < min(s0 + kElemTile, S.L); s += blockDim.x) {
+  const int s0 = it.idx * kGatherTile;
+  for (int s = s0 + threadIdx.x; s < min(s0 + kGatherTile, S.L); s += blockDim.x) {
     float al = 0.f, ar = 0.f;
     for (int r = 0; r < nres; ++r) {
       const LossRes& R = resv[r];
@@ -260,7 +372,12 @@ void launch_loss_frames(const LaunchCtx& c, const SongDev* songs, const LossRes*
                         int mode, int max_dy) {
   if (!n) return;
   const size_t smem = kFrameBuf * sizeof(float2) + (mode == 2 ? (size_t)max_dy * sizeof(float) : 0);
-  k_loss_frames<<<n, kLossThreads, smem, c.stream>>>(c, songs, res, items, mode);
+  switch (mode) {
+    case 0: k_loss_frames<0><<<n, kLossThreads, smem, c.stream>>>(c, songs, res, items); break;
+    case 1: k_loss_frames<1><<<n, kLossThreads, smem, c.stream>>>(c, songs, res, items); break;
+    case 2: k_loss_frames<2><<<n, kLossThreads, smem, c.stream>>>(c, songs, res, items); break;
+    default: k_loss_frames<3><<<n, kLossThreads, smem, c.stream>>>(c, songs, res, items);
+  }
 }
 
 void launch_loss_gather(const LaunchCtx& c, const SongDev* songs, const LossRes* res, int nres, const Item* items,
@@ -269,8 +386,12 @@ void launch_loss_gather(const LaunchCtx& c, const SongDev* songs, const LossRes*
 }
 
 void init_loss_attributes() {
-  cudaFuncSetAttribute(k_loss_frames, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kFrameBuf * sizeof(float2) + kLossMaxDy * sizeof(float));
+  const int frames = kFrameBuf * sizeof(float2);
+  cudaFuncSetAttribute(k_loss_frames<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, frames);
+  cudaFuncSetAttribute(k_loss_frames<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, frames);
+  cudaFuncSetAttribute(k_loss_frames<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       frames + kLossMaxDy * (int)sizeof(float));
+  cudaFuncSetAttribute(k_loss_frames<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, frames);
 }
 
 }  // namespace mg
