@@ -60,7 +60,7 @@ struct HostProc {
   // arena offsets (bytes)
   size_t o_cflag = 0;        // published states of the chained scans (c, n)
   size_t o_y = 0, o_stats = 0, o_fpart = 0, o_bpart = 0, o_taps = 0, o_dtaps = 0, o_aux = 0, o_carry = 0,
-         o_cagg = 0, o_nspec = 0, o_hspec = 0, o_ybar = 0, o_dhspec = 0, o_eqg = 0;
+         o_nspec = 0, o_hspec = 0, o_ybar = 0, o_dhspec = 0, o_eqg = 0;
   size_t scratch_bytes = 0;  // T1 + T2 + Hz
   size_t o_scratch = 0;      // offset inside the shared LTI scratch
 };
@@ -187,7 +187,7 @@ struct mg_console {
   size_t o_zero = 0;
   int score_mode = 0;              // 0: batched candidate scoring, 1: one full masked render per candidate
   int elem_tile = kElemTile;       // samples per work item of the elementwise kernels and sums (packing tuner)
-  unsigned* d_chain = nullptr;     // launch generation and work ticket of the chained scans
+  unsigned long long* d_chain = nullptr;   // chained scans: work ticket (low half) and launch generation (high half)
   int* h_err = nullptr;            // host-mapped error word of the chained scans' bounded waits
   int* d_err = nullptr;
   int chain_hold = 0;              // test hook (mg_debug_chain_hold)
@@ -986,7 +986,6 @@ void fill_procdev(mg_console* c, int pi) {
   }
   d.aux = p.o_aux ? (float*)A(p.o_aux) : nullptr;
   d.carry = p.nchunks ? (float*)A(p.o_carry) : nullptr;
-  d.chunkagg = p.nchunks ? (float*)A(p.o_cagg) : nullptr;
   d.cflag = p.nchunks ? (unsigned long long*)A(p.o_cflag) : nullptr;
   d.nchunks = p.nchunks;
   d.nspec = p.type == T_R ? (const float2*)A(p.o_nspec) : nullptr;
@@ -1391,9 +1390,8 @@ size_t layout_arena(mg_console* c, const mg_console_desc* d, size_t* shared_scra
       p.o_nspec = b.take((size_t)2 * p.nframes * kRevBins * sizeof(float2));
     }
     if (p.nchunks) {
-      p.o_cflag = b.take(p.nchunks * sizeof(unsigned long long));
+      p.o_cflag = b.take((size_t)2 * p.nchunks * sizeof(unsigned long long));
       p.o_carry = b.take(p.nchunks * sizeof(float));
-      p.o_cagg = b.take(p.nchunks * sizeof(float));
     }
   }
   if (c->is_graph) {
@@ -1722,8 +1720,11 @@ mg_status create_impl(mg_console* c, const mg_console_desc* d, const mg_song_des
   CK(cudaMalloc(&c->d_alphas, 4 * sizeof(float)));
   CK(cudaMalloc(&c->d_mask, std::max(1, c->P)));
   CK(cudaMalloc(&c->d_scratch_la, sizeof(float) * std::max<size_t>(1, c->songs.size())));
-  CK(cudaMalloc(&c->d_chain, 2 * sizeof(unsigned)));
-  CK(cudaMemsetAsync(c->d_chain, 0, 2 * sizeof(unsigned), c->stream));
+  CK(cudaMalloc(&c->d_chain, sizeof(unsigned long long)));
+  {
+    const unsigned long long first = 1ull << 32;   // ticket 0 of generation 1 (cleared flags hold generation 0)
+    CK(cudaMemcpy(c->d_chain, &first, sizeof(first), cudaMemcpyHostToDevice));
+  }
   CK(cudaHostAlloc(&c->h_err, sizeof(int), cudaHostAllocMapped));
   *c->h_err = 0;
   CK(cudaHostGetDevicePointer(&c->d_err, c->h_err, 0));
@@ -2114,7 +2115,7 @@ size_t copy_bytes(const mg_console* c, int pi, size_t* items) {
   size_t it = 0;
   if (p.nfrows) b += al((size_t)std::max(p.nfrows, p.nfcap) * kNPart * sizeof(float));
   if (p.type == T_C || p.type == T_N) {
-    b += 2 * al((size_t)p.nchunks * sizeof(float)) + (size_t)p.nchunks * sizeof(unsigned long long) +
+    b += al((size_t)p.nchunks * sizeof(float)) + (size_t)2 * p.nchunks * sizeof(unsigned long long) +
          sizeof(CUtensorMap);   // + states, + tensor map
     it = p.nchunks + 1;
   } else if (p.type == T_G || p.type == T_S) {
@@ -2269,9 +2270,8 @@ void build_chunk(mg_console* c, const std::vector<CandPlan>& plans, const uint8_
         d.ybar = p.type == T_E ? (float*)w.buffer((size_t)2 * p.ld * sizeof(float)) : nullptr;
         if (p.type == T_C || p.type == T_N) {
           d.carry = (float*)w.buffer((size_t)p.nchunks * sizeof(float));
-          d.chunkagg = (float*)w.buffer((size_t)p.nchunks * sizeof(float));
           d.aux = nullptr;
-          flag_nodes.push_back({(int)k.vp.size(), p.nchunks});
+          flag_nodes.push_back({(int)k.vp.size(), 2 * p.nchunks});
           d.umap = nullptr;
           d.dymap = nullptr;
           CUtensorMap m;
@@ -2461,8 +2461,7 @@ std::string check_chunk(const mg_console* c, const ScoreChunk& k) {
     if (d.fpart && !in(d.fpart, (size_t)d.nfpart * kNPart * sizeof(float)))
       return "node copy " + std::to_string(v) + ": partials out of range";
     if ((d.type == T_C || d.type == T_N) &&
-        (!in(d.carry, (size_t)d.nchunks * 4) || !in(d.chunkagg, (size_t)d.nchunks * 4) ||
-         !in(d.cflag, (size_t)d.nchunks * 8)))
+        (!in(d.carry, (size_t)d.nchunks * 4) || !in(d.cflag, (size_t)d.nchunks * 16)))
       return "node copy " + std::to_string(v) + ": scan carries out of range";
     if (d.type == T_R || d.type == T_D) {
       const size_t N = (size_t)d.f << d.logN;

@@ -4,9 +4,13 @@
 // taken earlier by a CTA that is running or finished.  A CTA
 //   1. computes its chunk's zero-start end state (a warp-shuffle scan of the per-thread states, decay alpha^16
 //      per thread),
-//   2. waits (bounded) for the state entering its chunk, published by the CTA of the previous chunk, and
-//      publishes the state entering the next chunk, g_next = A g_in + agg (A = alpha^4096); the stage's chunks are
-//      listed in rounds across nodes, so that wait is normally over before it starts,
+//   2. publishes that end state at once, then looks back (bounded) over the 32 chunks before it for the nearest one
+//      whose leaving state is known and steps from there, g <- A g + agg (A = alpha^4096) over the end states of the
+//      chunks between: the same multiply-adds in the same order wherever the walk starts, so the state's bits do not
+//      depend on timing; then publishes the state that leaves its own chunk.  The stage's chunks are listed in rounds
+//      across nodes, so on a batch the previous chunk's state is normally there already; on one song, whose nodes do
+//      not fill the GPU, the chain is a hop per 32 chunks instead of one per chunk (a stage of 16 nodes x 10 s took 83 us forward and
+//      103 us backward, now 28 and 63; 8 nodes x 60 s 420 and 480 us, now 70 and 170),
 //   3. rescans its chunk from that state and applies the gain law (Eqs. 13-16) and Eq. (15), fused with the
 //      dry/wet blend.  The forward's input arrives by TMA (a bulk tensor copy into shared memory, read by both
 //      steps) when the node has a tensor map, else by plain loads with the rescan from L2.
@@ -189,48 +193,59 @@ __device__ __forceinline__ float scan_rev_excl(float r, const float* dl, const f
 
 constexpr long long kChainWaitCycles = 1000000000LL;   // about half a second at the SM clock
 
-__global__ void k_chain_begin(unsigned* chain) {
-  chain[0] += 1u;   // a new launch generation: flags of earlier launches no longer match
-  chain[1] = 0u;    // the work ticket
-}
-
-// Work item of this CTA in ticket order (thread 0 draws, the block reads it after the barrier).
+// Work item of this CTA in ticket order and the launch generation: one 64-bit word holds the ticket (low) and the
+// generation (high), so a draw reads both at once; the draw of the last item starts the next launch's generation
+// (every ticket of this launch is out by then, and the next launch on the stream starts after this one).
 __device__ __forceinline__ Item take_item(const LaunchCtx& c, const Item* items, int* s_idx, unsigned* s_gen) {
   if (threadIdx.x == 0) {
-    *s_idx = (int)atomicAdd(&c.chain[1], 1u);
-    *s_gen = *(volatile unsigned*)&c.chain[0];
+    const unsigned long long w = atomicAdd(c.chain, 1ull);
+    *s_idx = (int)(unsigned)w;
+    *s_gen = (unsigned)(w >> 32);
+    if ((unsigned)w == gridDim.x - 1) *(volatile unsigned long long*)c.chain = ((w >> 32) + 1ull) << 32;
   }
   __syncthreads();
   return items[*s_idx];
 }
 
-// Thread 0: the state entering chunk k (0 for the first chunk of the direction), once the CTA of the neighbouring
-// chunk has published it; then the state entering the next chunk, published for its CTA.  A published state is one
-// 64-bit word, the launch generation in the high half and the float's bits in the low half, written and read as a
-// whole: the value arrives with its flag, and no fence is needed between them.  keep (forward only) receives the
-// state entering chunk k for the backward.
-__device__ __forceinline__ float chain_link(const LaunchCtx& c, const ProcDev& P, int k, int next, bool first,
-                                            float agg, float A, unsigned gen, bool hold, float* keep) {
+// Warp 0, every lane: the state entering chunk k of the direction dir (+1 forward, -1 backward; 0 for the first
+// chunk).  A published value is one 64-bit word, the launch generation in the high half and the float's bits in the
+// low half, written and read as a whole: the value arrives with its flag, and no fence is needed between them.
+// cflag[q] holds the state leaving chunk q, cflag[nchunks + q] its zero-start end state.  keep (forward only)
+// receives the state entering chunk k for the backward.
+__device__ __forceinline__ float chain_link(const LaunchCtx& c, const ProcDev& P, int k, int dir, float agg, float A,
+                                            unsigned gen, bool hold, float* keep) {
+  const int lane = threadIdx.x & 31, n = P.nchunks, pos = dir > 0 ? k : n - 1 - k;
+  volatile unsigned long long* leave = P.cflag;
+  volatile unsigned long long* ends = P.cflag + n;
+  auto word = [&](float v) { return ((unsigned long long)gen << 32) | __float_as_uint(v); };
+  if (lane == 0 && !hold) ends[k] = word(agg);
   float in = 0.f;
-  if (!first) {
-    volatile unsigned long long* f = P.cflag + k;
+  if (pos > 0) {
+    const int q = k - dir * (lane + 1);     // this lane's chunk before k; at and beyond the start the state is 0
+    const bool real = lane < pos;
     const long long t0 = clock64();
-    unsigned long long w = *f;
-    while ((unsigned)(w >> 32) != gen) {
-      if (clock64() - t0 > kChainWaitCycles) {
-        *(volatile int*)c.err = 1;
-        w = 0ull;   // continue from a zero state
+    while (true) {
+      const unsigned long long wl = real ? leave[q] : 0ull, we = real ? ends[q] : 0ull;
+      const unsigned known = __ballot_sync(0xffffffffu, !real || (unsigned)(wl >> 32) == gen);
+      const unsigned ended = __ballot_sync(0xffffffffu, real && (unsigned)(we >> 32) == gen);
+      const int from = known ? __ffs(known) - 1 : 32;
+      const unsigned between = from < 32 ? (1u << from) - 1u : 0xffffffffu;
+      if (from < 32 && (ended & between) == between) {
+        in = __shfl_sync(0xffffffffu, __uint_as_float((unsigned)wl), from);
+        for (int l = from - 1; l >= 0; --l) in = fmaf(A, in, __shfl_sync(0xffffffffu, __uint_as_float((unsigned)we), l));
         break;
       }
+      if (__any_sync(0xffffffffu, clock64() - t0 > kChainWaitCycles)) {
+        if (lane == 0) *(volatile int*)c.err = 1;
+        break;   // continue from a zero state
+      }
       __nanosleep(32);
-      w = *f;
     }
-    in = __uint_as_float((unsigned)w);
   }
-  if (next >= 0 && next < P.nchunks && !hold)
-    *(volatile unsigned long long*)(P.cflag + next) =
-        ((unsigned long long)gen << 32) | __float_as_uint(fmaf(A, in, agg));
-  if (keep) keep[k] = in;
+  if (lane == 0) {
+    if (!hold) leave[k] = word(fmaf(A, in, agg));
+    if (keep) keep[k] = in;
+  }
   return in;
 }
 
@@ -348,9 +363,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_dyn_fwd(LaunchCtx c, const Item
   float v[1] = {s * (dec[31 - (t & 31)] * dec[32 + 7 - (t >> 5)])};   // alpha^(16 (255 - t))
   float out[1];
   block_sum<1>(v, red, out);
-  if (t == 0) {
-    const float A = expf((float)kDynChunk * d.lna);
-    s_in = chain_link(c, P, it.idx, it.idx + 1, it.idx == 0, out[0], A, s_gen, c.chain_hold && s_idx == 0, P.carry);
+  if (t < 32) {
+    const float A = expf((float)kDynChunk * d.lna), agg = __shfl_sync(0xffffffffu, out[0], 0);
+    const float in = chain_link(c, P, it.idx, 1, agg, A, s_gen, c.chain_hold && s_idx == 0, P.carry);
+    if (t == 0) s_in = in;
   }
   __syncthreads();
   const float w = dry_wet_w(c, P.qidx), wd = dry_wet_d(c, P.qidx);
@@ -494,13 +510,15 @@ __global__ void __launch_bounds__(kThreads, 3) k_dyn_bwd(LaunchCtx c, const Item
     float v[5] = {lam * (dec[t & 31] * dec[32 + (t >> 5)]), acc.dT, acc.dW, acc.dR, acc.dw};
     float out[5];
     block_sum<5>(v, sm, out);
-    if (t == 0) {
-      float* bp = P.bpart + (size_t)it.idx * kNPart;
+    if (t < 32) {
+      const float A = expf((float)kDynChunk * d.lna), agg = __shfl_sync(0xffffffffu, out[0], 0);
+      const float in = chain_link(c, P, it.idx, -1, agg, A, s_gen, c.chain_hold && s_idx == 0, nullptr);
+      if (t == 0) {
+        s_in = in;
+        float* bp = P.bpart + (size_t)it.idx * kNPart;
 #pragma unroll
-      for (int j = 1; j < 5; ++j) bp[j] = out[j];
-      const float A = expf((float)kDynChunk * d.lna);
-      s_in = chain_link(c, P, it.idx, it.idx - 1, it.idx == P.nchunks - 1, out[0], A, s_gen,
-                        c.chain_hold && s_idx == 0, nullptr);
+        for (int j = 1; j < 5; ++j) bp[j] = out[j];
+      }
     }
   }
   __syncthreads();   // this CTA's du and aux stores are visible to its own loads below
@@ -564,12 +582,10 @@ void init_dyn_attributes() {
 
 void launch_dyn_fwd(const LaunchCtx& c, const Item* items, int n) {
   if (!n) return;
-  k_chain_begin<<<1, 1, 0, c.stream>>>(c.chain);
   k_dyn_fwd<<<n, kThreads, c.dyn_tma ? kDynFwdSmem : 0, c.stream>>>(c, items);   // no stage without maps
 }
 void launch_dyn_bwd(const LaunchCtx& c, const Item* items, int n) {
   if (!n) return;
-  k_chain_begin<<<1, 1, 0, c.stream>>>(c.chain);
   k_dyn_bwd<<<n, kThreads, c.dyn_tma ? kDynBwdSmem : 0, c.stream>>>(c, items);
 }
 

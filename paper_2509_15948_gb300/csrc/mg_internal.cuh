@@ -79,8 +79,8 @@ struct ProcDev {
                                            // compressor, noisegate: dL/dg per sample)
   // envelope scans (c, n)
   float* carry;                            // [nchunks] forward state entering each chunk
-  float* chunkagg;                         // [nchunks] per-chunk aggregates
-  unsigned long long* cflag;               // [nchunks] chained-scan states: launch generation << 32 | state bits
+  unsigned long long* cflag;               // [2][nchunks] chained-scan states leaving each chunk, then the chunks'
+                                           // zero-start end states: launch generation << 32 | state bits
   const void* umap;                        // c, n: tensor map (TMA) of u as rows of 32 floats, or nullptr
   const void* dymap;                       // c, n: the same of dL/dy (backward), or nullptr
   int nchunks;
@@ -151,7 +151,7 @@ struct LaunchCtx {
   float alpha_g;
   double fs;
   int elem_tile;                           // samples per work item of the gain/pan and imager kernels
-  unsigned* chain;                         // device [2]: launch generation and work ticket of the chained scans
+  unsigned long long* chain;               // device: work ticket and launch generation of the chained scans
   int* err;                                // host-mapped error word: 1 = a chained scan's wait ran out
   int chain_hold;                          // test hook: the first work item does not publish its state
   int dyn_tma;                             // the scans' nodes may carry tensor maps (their launches reserve the stage)
