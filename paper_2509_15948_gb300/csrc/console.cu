@@ -34,12 +34,12 @@ constexpr int kParamCount[NTYPES] = {1024, 4, 4, 1, 2, 880, 768};
 enum Family {
   F_GS_FWD, F_GS_BWD, F_SUM, F_DYN_FWD, F_DYN_BWD, F_EQ_FIR, F_DLY_FIR, F_REV_FIR, F_FIR_ADJ, F_COL_FWD, F_ROW_HZ,
   F_ROW_CONV, F_COL_OUT, F_COL_DYBAR, F_ROW_BWD2, F_COL_DU, F_COL_DH, F_LOSS_FWD, F_LOSS_BWD, F_LOSS_GATHER,
-  F_FINALIZE, F_ADAM, F_MISC, F_EQ_OS_FWD, F_EQ_OS_BWD, F_EQ_OS_DU, F_SCALE, F_COUNT
+  F_FINALIZE, F_ADAM, F_MISC, F_EQ_OS_FWD, F_EQ_OS_BWD, F_SCALE, F_COUNT
 };
 const char* kFamilyNames[F_COUNT] = {
     "gs_fwd", "gs_bwd", "sum", "dyn_fwd", "dyn_bwd", "eq_fir", "dly_fir", "rev_fir", "fir_adj", "col_fwd", "row_hz",
     "row_conv", "col_out", "col_dybar", "row_bwd2", "col_du", "col_dh", "loss_fwd", "loss_bwd", "loss_gather",
-    "finalize", "adam", "misc", "eq_os_fwd", "eq_os_bwd", "eq_os_du", "chan_scale"};
+    "finalize", "adam", "misc", "eq_os_fwd", "eq_os_bwd", "chan_scale"};
 
 inline int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 inline int ilog2_ceil(int64_t x) {
@@ -60,7 +60,7 @@ struct HostProc {
   // arena offsets (bytes)
   size_t o_cflag = 0;        // published states of the chained scans (c, n)
   size_t o_y = 0, o_stats = 0, o_fpart = 0, o_bpart = 0, o_taps = 0, o_dtaps = 0, o_aux = 0, o_carry = 0,
-         o_nspec = 0, o_hspec = 0, o_ybar = 0, o_dhspec = 0, o_eqg = 0;
+         o_nspec = 0, o_hspec = 0, o_ybar = 0, o_eqg = 0;
   size_t scratch_bytes = 0;  // T1 + T2 + Hz
   size_t o_scratch = 0;      // offset inside the shared LTI scratch
 };
@@ -121,7 +121,7 @@ struct Stage {
   ItemList elem;                 // g, s, c, n (tile / chunk items)
   ItemList elem_rev;             // c, n: chunk items in reverse order per node (the chained backward)
   ItemList chain_f, chain_b;     // c, n: the same chunks in rounds across nodes (batched launches)
-  ItemList osf, osb;             // e: overlap-save blocks of the forward and backward kernels
+  ItemList osf;                  // e: overlap-save blocks
   std::vector<LtiGroup> groups;  // e, r, d
 };
 
@@ -364,7 +364,7 @@ void size_proc(HostProc& p, double fs) {
     p.colG = std::min(8, std::min(8192 >> p.logN2, 1 << p.logN1));
     if (t == T_E) {   // single-pass overlap-save in shared memory (no global FFT scratch)
       p.nfrows = (p.L + kEqOsFwdBlock - 1) / kEqOsFwdBlock;
-      p.nbrows = (p.nfrows + kEqChunk - 1) / kEqChunk;   // backward items: chunks of forward blocks
+      p.nbrows = p.nfrows;
     } else {
       p.nfrows = (p.f << p.logN1) / p.colG;
       p.nbrows = p.nfrows;
@@ -759,8 +759,7 @@ void stage_backward(mg_console* c, const LaunchCtx& x, Stage& s) {
       run_items(c, F_DYN_BWD, c->per_node ? s.elem_rev : s.chain_b, [&](const Item* it, int n) { launch_dyn_bwd(x, it, n); });
       break;
     case T_E:
-      run_items(c, F_EQ_OS_BWD, s.osb, [&](const Item* it, int n) { launch_eq_os_bwd(x, it, n); });
-      run_items(c, F_EQ_OS_DU, s.osf, [&](const Item* it, int n) { launch_eq_os_du(x, it, n); });
+      run_items(c, F_EQ_OS_BWD, s.osf, [&](const Item* it, int n) { launch_eq_os_bwd(x, it, n); });
       run_procs(c, F_FIR_ADJ, s.procs, [&](const int* p, int n) { launch_eq_dh_reduce(x, p, n); });
       run_procs(c, F_FIR_ADJ, s.procs, [&](const int* p, int n) { launch_eq_fir_adj(x, p, n); });
       break;
@@ -981,7 +980,6 @@ void fill_procdev(mg_console* c, int pi) {
   if (p.type == T_E) {
     d.hspec = (float*)A(p.o_hspec);
     d.ybar = (float*)A(p.o_ybar);
-    d.dhspec = (float2*)A(p.o_dhspec);
     d.eqg = (float2*)A(p.o_eqg);
   }
   d.aux = p.o_aux ? (float*)A(p.o_aux) : nullptr;
@@ -1033,16 +1031,13 @@ mg_status make_stage(mg_console* c, Stage& st) {
         upload_items(c, st.chain_b) || upload_procs(c, st.procs))
       return MG_ERR_CUDA;
   } else if (t == T_E) {
-    // equalizer: overlap-save blocks (forward and backward blockings differ)
+    // equalizer: overlap-save blocks
     for (int pi : st.procs.h) {
       st.osf.beg.push_back((int)st.osf.h.size());
-      st.osb.beg.push_back((int)st.osb.h.size());
       for (int i = 0; i < c->procs[pi].nfrows; ++i) st.osf.h.push_back(Item{pi, i});
-      for (int i = 0; i < c->procs[pi].nbrows; ++i) st.osb.h.push_back(Item{pi, i});
     }
     st.osf.beg.push_back((int)st.osf.h.size());
-    st.osb.beg.push_back((int)st.osb.h.size());
-    if (upload_items(c, st.osf) || upload_items(c, st.osb) || upload_procs(c, st.procs)) return MG_ERR_CUDA;
+    if (upload_items(c, st.osf) || upload_procs(c, st.procs)) return MG_ERR_CUDA;
   } else {
     // LTI: groups under the workspace limit, each with its own scratch offsets
     size_t used = 0;
@@ -1379,7 +1374,6 @@ size_t layout_arena(mg_console* c, const mg_console_desc* d, size_t* shared_scra
     if (p.type == T_E) {
       p.o_hspec = b.take((size_t)kEqOsM * sizeof(float));
       p.o_ybar = b.take((size_t)2 * p.ld * sizeof(float));
-      p.o_dhspec = b.take((size_t)p.nbrows * kEqOsM * sizeof(float2));
       p.o_eqg = b.take((size_t)p.nfrows * kEqOsM * sizeof(float2));
     }
     if (p.type == T_D) p.o_aux = b.take((2 * kDlyTaps * kDlyFir + 2 * kDlyTaps) * sizeof(float));
@@ -2265,7 +2259,6 @@ void build_chunk(mg_console* c, const std::vector<CandPlan>& plans, const uint8_
         d.gp = nullptr;
         d.bpart = nullptr;
         d.dtaps = nullptr;
-        d.dhspec = nullptr;
         d.eqg = nullptr;
         d.ybar = p.type == T_E ? (float*)w.buffer((size_t)2 * p.ld * sizeof(float)) : nullptr;
         if (p.type == T_C || p.type == T_N) {

@@ -41,7 +41,6 @@ constexpr int kEvalPiece = 16384;          // samples per evaluation piece (two 
 constexpr int kEvalPart = 40, kEvalSeg = 8;  // doubles per evaluation work item / per segment
 constexpr int kEqOsM = 8192;               // overlap-save FFT size of the equalizer
 constexpr int kEqOsFwdBlock = kEqOsM - 2 * kEqHalf;        // 6146 outputs per forward block
-constexpr int kEqChunk = 8;                 // equalizer backward: blocks per work item (spectra summed in registers)
 
 struct Item {
   int proc;
@@ -90,8 +89,7 @@ struct ProcDev {
   // equalizer (overlap-save)
   float* hspec;                            // [8192] real spectrum of the FIR on the overlap-save grid
   float* ybar;                             // [2][ld] wet signal kept by the forward for the backward
-  float2* dhspec;                          // [backward items][8192] summed spectra of the tap correlation
-  float2* eqg;                             // [forward blocks][8192] spectra D H of the equalizer backward
+  float2* eqg;                             // [blocks][8192] spectra of the tap correlation (equalizer backward)
 };
 
 struct LossRes {                           // one STFT resolution of Eq. (21)
@@ -188,7 +186,6 @@ void init_eqos_attributes();
 void launch_eq_spec(const LaunchCtx&, const int* procs, int n);
 void launch_eq_os_fwd(const LaunchCtx&, const Item* items, int n);
 void launch_eq_os_bwd(const LaunchCtx&, const Item* items, int n);
-void launch_eq_os_du(const LaunchCtx&, const Item* items, int n);
 void launch_eq_dh_reduce(const LaunchCtx&, const int* procs, int n);
 void launch_col_fwd_audio(const LaunchCtx&, const Item* items, int n, int maxN2G);
 void launch_col_fwd_taps(const LaunchCtx&, const Item* items, int n, int maxN2G);
