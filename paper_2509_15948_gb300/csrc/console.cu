@@ -208,6 +208,14 @@ struct mg_console {
   std::vector<LossRes> hres;
   int loss_max_dy = 0;            // floats of the loss adjoint's per-item band gradients (largest resolution)
   std::vector<Stage> stages;      // forward order
+  // parameter-only work of every present e, d, r processor (all stages of a type together): FIR synthesis and, where
+  // the spectra are kept, the filters' transforms
+  LtiGroup fir[3];
+  // its streams and events (see fir_synthesis): [0] delays and equalizers, [1] reverbs
+  cudaStream_t side[2] = {nullptr, nullptr};
+  cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr};
+  bool fir_pending[2] = {false, false};   // this render's synthesis that the main stream has not waited for yet
+  bool adj_pending[2] = {false, false};   // this backward's adjoints, the same
   // sums
   DevVec<float*> sum_out;
   DevVec<const float*> sum_in;
@@ -684,17 +692,69 @@ LaunchCtx make_ctx(mg_console* c, const uint8_t* mask) {
   return x;
 }
 
-void lti_forward(mg_console* c, const LaunchCtx& x, int type, LtiGroup& g) {
-  if (type == T_E) run_procs(c, F_EQ_FIR, g.procs, [&](const int* p, int n) { launch_eq_fir(x, p, n); });
-  if (type == T_D) {
-    run_procs(c, F_DLY_FIR, g.procs, [&](const int* p, int n) { launch_dly_prep(x, p, n); });
-    run_items(c, F_DLY_FIR, g.firtaps, [&](const Item* it, int n) { launch_dly_fir(x, it, n); });
+// The work of a pass that only parameters feed (FIR synthesis, the kept filter spectra) or that only feeds parameter
+// gradients (dL/dh and the FIR adjoints) runs on two side streams beside the chain of audio kernels: on a small console
+// it was two thirds of the launches and half of the time, a few CTAs each.  4 tracks x 2 s step 1,153 -> 878 us,
+// 16 x 10 s 3,880 -> 3,558 us.  Every pass forks from the console's stream and joins it before it returns, so callers
+// see one stream.  Everything stays on the console's stream for one launch per node, per-launch timing and
+// MG_DEBUG_SYNC.
+bool overlapped(const mg_console* c) { return !c->per_node && !c->profiling && !c->debug_sync; }
+int side_of(int type) { return type == T_R ? 1 : 0; }
+int fir_slot(int type) { return type == T_E ? 0 : (type == T_D ? 1 : 2); }
+
+// x on the side stream of a type, which waits for everything issued on the console's stream so far
+LaunchCtx fork(mg_console* c, const LaunchCtx& x, int type, bool* pending) {
+  if (!overlapped(c)) return x;
+  LaunchCtx y = x;
+  y.stream = c->side[side_of(type)];
+  cudaEventRecord(c->ev_fork, c->stream);
+  cudaStreamWaitEvent(y.stream, c->ev_fork, 0);
+  pending[side_of(type)] = true;
+  return y;
+}
+
+// The console's stream waits for what a fork left pending on a side stream.
+void join(mg_console* c, int side, bool* pending) {
+  if (!pending[side]) return;
+  cudaEventRecord(c->ev_join[side], c->side[side]);
+  cudaStreamWaitEvent(c->stream, c->ev_join[side], 0);
+  pending[side] = false;
+}
+
+// FIR synthesis of all nodes.  The equalizers come first in a chain: their FIRs stay on the console's stream.
+void fir_synthesis(mg_console* c, const LaunchCtx& x) {
+  for (int type : {T_D, T_R}) {
+    LtiGroup& g = c->fir[fir_slot(type)];
+    if (g.procs.h.empty()) continue;
+    StageScope scope(c, type);
+    const LaunchCtx y = fork(c, x, type, c->fir_pending);
+    if (type == T_D) {
+      run_procs(c, F_DLY_FIR, g.procs, [&](const int* p, int n) { launch_dly_prep(y, p, n); });
+      run_items(c, F_DLY_FIR, g.firtaps, [&](const Item* it, int n) { launch_dly_fir(y, it, n); });
+    } else {
+      run_items(c, F_REV_FIR, g.revfir, [&](const Item* it, int n) { launch_rev_fir(y, it, n); });
+    }
+    run_procs(c, F_SCALE, g.procs, [&](const int* p, int n) { launch_chan_scale(y, p, n, kScaleOfTaps); });
+    if (c->retain) {
+      run_items(c, F_COL_FWD, g.col, [&](const Item* it, int n) { launch_col_fwd_taps(y, it, n, g.col.maxv); });
+      run_items(c, F_ROW_HZ, g.rowpair, [&](const Item* it, int n) { launch_row_fwd_hz(y, it, n, g.rowpair.maxv); });
+    }
   }
-  if (type == T_R) run_items(c, F_REV_FIR, g.revfir, [&](const Item* it, int n) { launch_rev_fir(x, it, n); });
-  run_procs(c, F_SCALE, g.procs, [&](const int* p, int n) { launch_chan_scale(x, p, n, 0); });
-  run_items(c, F_COL_FWD, g.col, [&](const Item* it, int n) { launch_col_fwd_taps(x, it, n, g.col.maxv); });
-  run_items(c, F_ROW_HZ, g.rowpair, [&](const Item* it, int n) { launch_row_fwd_hz(x, it, n, g.rowpair.maxv); });
+  LtiGroup& g = c->fir[fir_slot(T_E)];
+  StageScope scope(c, T_E);
+  run_procs(c, F_EQ_FIR, g.procs, [&](const int* p, int n) { launch_eq_fir(x, p, n); });
+  run_procs(c, F_EQ_FIR, g.procs, [&](const int* p, int n) { launch_eq_spec(x, p, n); });
+}
+
+void lti_forward(mg_console* c, const LaunchCtx& x, int type, LtiGroup& g) {
+  run_procs(c, F_SCALE, g.procs, [&](const int* p, int n) { launch_chan_scale(x, p, n, kScaleOfInput); });
+  if (!c->retain) {   // one scratch for all stages: the filters' transforms wait for their turn
+    join(c, side_of(type), c->fir_pending);
+    run_items(c, F_COL_FWD, g.col, [&](const Item* it, int n) { launch_col_fwd_taps(x, it, n, g.col.maxv); });
+    run_items(c, F_ROW_HZ, g.rowpair, [&](const Item* it, int n) { launch_row_fwd_hz(x, it, n, g.rowpair.maxv); });
+  }
   run_items(c, F_COL_FWD, g.col, [&](const Item* it, int n) { launch_col_fwd_audio(x, it, n, g.col.maxv); });
+  join(c, side_of(type), c->fir_pending);
   if (c->retain) {   // U stays in T1, y_bar in T2 (natural order) for the backward
     run_items(c, F_ROW_CONV, g.rowpair, [&](const Item* it, int n) { launch_row_conv_fwd(x, it, n, g.rowpair.maxv, true); });
     run_items(c, F_COL_OUT, g.col, [&](const Item* it, int n) { launch_col_inv_out_keep(x, it, n, g.col.maxv); });
@@ -705,7 +765,7 @@ void lti_forward(mg_console* c, const LaunchCtx& x, int type, LtiGroup& g) {
 }
 
 void lti_backward(mg_console* c, const LaunchCtx& x, int type, LtiGroup& g) {
-  run_procs(c, F_SCALE, g.procs, [&](const int* p, int n) { launch_chan_scale(x, p, n, 1); });
+  run_procs(c, F_SCALE, g.procs, [&](const int* p, int n) { launch_chan_scale(x, p, n, kScaleOfAdjoint); });
   if (c->retain) {
     run_items(c, F_COL_DYBAR, g.col, [&](const Item* it, int n) { launch_col_dybar_keep(x, it, n, g.col.maxv); });
   } else {
@@ -716,14 +776,18 @@ void lti_backward(mg_console* c, const LaunchCtx& x, int type, LtiGroup& g) {
     run_items(c, F_COL_DYBAR, g.col, [&](const Item* it, int n) { launch_col_dybar(x, it, n, g.col.maxv); });
   }
   run_items(c, F_ROW_BWD2, g.rowpair, [&](const Item* it, int n) { launch_row_bwd2(x, it, n, g.rowpair.maxv); });
-  run_items(c, F_COL_DU, g.col, [&](const Item* it, int n) { launch_col_du(x, it, n, g.col.maxv); });
-  run_items(c, F_COL_DH, g.col, [&](const Item* it, int n) { launch_col_dh(x, it, n, g.col.maxv); });
-  if (type == T_E) run_procs(c, F_FIR_ADJ, g.procs, [&](const int* p, int n) { launch_eq_fir_adj(x, p, n); });
-  if (type == T_D) run_items(c, F_FIR_ADJ, g.dlyadj, [&](const Item* it, int n) { launch_dly_adj(x, it, n); });
+  // dL/dh and the FIR adjoint beside the chain; without kept spectra dL/dh reads the scratch that the next stage
+  // writes, so only the adjoint leaves the console's stream
+  LaunchCtx y = x;
+  if (c->retain) y = fork(c, x, type, c->adj_pending);
+  run_items(c, F_COL_DH, g.col, [&](const Item* it, int n) { launch_col_dh(y, it, n, g.col.maxv); });
+  if (!c->retain) y = fork(c, x, type, c->adj_pending);
+  if (type == T_D) run_items(c, F_FIR_ADJ, g.dlyadj, [&](const Item* it, int n) { launch_dly_adj(y, it, n); });
   if (type == T_R) {
-    run_items(c, F_FIR_ADJ, g.revfir, [&](const Item* it, int n) { launch_rev_adj(x, it, n); });
-    run_procs(c, F_FIR_ADJ, g.procs, [&](const int* p, int n) { launch_rev_adj_fin(x, p, n); });
+    run_items(c, F_FIR_ADJ, g.revfir, [&](const Item* it, int n) { launch_rev_adj(y, it, n); });
+    run_procs(c, F_FIR_ADJ, g.procs, [&](const int* p, int n) { launch_rev_adj_fin(y, p, n); });
   }
+  run_items(c, F_COL_DU, g.col, [&](const Item* it, int n) { launch_col_du(x, it, n, g.col.maxv); });
 }
 
 void stage_forward(mg_console* c, const LaunchCtx& x, Stage& s) {
@@ -738,8 +802,6 @@ void stage_forward(mg_console* c, const LaunchCtx& x, Stage& s) {
       run_items(c, F_DYN_FWD, c->per_node ? s.elem : s.chain_f, [&](const Item* it, int n) { launch_dyn_fwd(x, it, n); });
       break;
     case T_E:
-      run_procs(c, F_EQ_FIR, s.procs, [&](const int* p, int n) { launch_eq_fir(x, p, n); });
-      run_procs(c, F_EQ_FIR, s.procs, [&](const int* p, int n) { launch_eq_spec(x, p, n); });
       run_items(c, F_EQ_OS_FWD, s.osf, [&](const Item* it, int n) { launch_eq_os_fwd(x, it, n); });
       break;
     default:
@@ -758,11 +820,14 @@ void stage_backward(mg_console* c, const LaunchCtx& x, Stage& s) {
     case T_N:
       run_items(c, F_DYN_BWD, c->per_node ? s.elem_rev : s.chain_b, [&](const Item* it, int n) { launch_dyn_bwd(x, it, n); });
       break;
-    case T_E:
+    case T_E: {
       run_items(c, F_EQ_OS_BWD, s.osf, [&](const Item* it, int n) { launch_eq_os_bwd(x, it, n); });
-      run_procs(c, F_FIR_ADJ, s.procs, [&](const int* p, int n) { launch_eq_dh_reduce(x, p, n); });
-      run_procs(c, F_FIR_ADJ, s.procs, [&](const int* p, int n) { launch_eq_fir_adj(x, p, n); });
+      // issued eagerly, the fork costs more than it hides (equalizer block 976 us with it, 922 without)
+      const LaunchCtx y = c->capturing ? fork(c, x, T_E, c->adj_pending) : x;
+      run_procs(c, F_FIR_ADJ, s.procs, [&](const int* p, int n) { launch_eq_dh_reduce(y, p, n); });
+      run_procs(c, F_FIR_ADJ, s.procs, [&](const int* p, int n) { launch_eq_fir_adj(y, p, n); });
       break;
+    }
     default:
       for (auto& g : s.groups) lti_backward(c, x, s.type, g);
   }
@@ -776,6 +841,7 @@ void run_sums(mg_console* c, const ItemList& items) {
 
 // Forward of a graph: per schedule step the aggregation sums, then the step's processors (Alg. 1).
 void render_graph(mg_console* c, const LaunchCtx& x) {
+  fir_synthesis(c, x);
   for (size_t k = 0; k < c->gstep_type.size(); ++k) {
     {
       StageScope scope(c, 8);
@@ -783,6 +849,7 @@ void render_graph(mg_console* c, const LaunchCtx& x) {
     }
     if (c->gstep_stage[k] >= 0) stage_forward(c, x, c->stages[c->gstep_stage[k]]);
   }
+  for (int i : {0, 1}) join(c, i, c->fir_pending);
 }
 
 void render(mg_console* c, const LaunchCtx& x) {
@@ -790,6 +857,7 @@ void render(mg_console* c, const LaunchCtx& x) {
     render_graph(c, x);
     return;
   }
+  fir_synthesis(c, x);
   for (int level = 0; level < 2; ++level) {
     if (level == 1 && !c->sum_m_items.h.empty()) {
       StageScope scope(c, 8);
@@ -800,6 +868,7 @@ void render(mg_console* c, const LaunchCtx& x) {
     for (auto& s : c->stages)
       if (s.level == level) stage_forward(c, x, s);
   }
+  for (int i : {0, 1}) join(c, i, c->fir_pending);
   StageScope scope(c, 8);
   run_items(c, F_SUM, c->sum_o_items, [&](const Item* it, int n) {
     launch_sum(c->stream, c->sum_out.d, c->sum_in.d, c->sum_beg.d, c->sum_L.d, c->sum_ld.d, it, n, c->elem_tile);
@@ -847,6 +916,7 @@ void backward_pass(mg_console* c, const LaunchCtx& x) {
   run_procs(c, F_FINALIZE, c->all_present, [&](const int* p, int n) { launch_node_stats(x, p, n, 0); });
   run_procs(c, F_FINALIZE, c->all_present,
             [&](const int* p, int n) { launch_grad_finalize2(x, p, n, c->d_grads + c->npp); });
+  for (int i : {0, 1}) join(c, i, c->adj_pending);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1090,6 +1160,36 @@ mg_status make_stage(mg_console* c, Stage& st) {
   return MG_OK;
 }
 
+// Lists of the parameter-only work: the stages' groups of one type joined.
+mg_status join_fir_lists(mg_console* c) {
+  for (int type : {T_E, T_D, T_R}) {
+    LtiGroup& f = c->fir[fir_slot(type)];
+    f = LtiGroup{};
+    auto append = [](ItemList& to, const ItemList& from) {
+      const int o = (int)to.h.size();
+      if (!to.beg.empty()) to.beg.pop_back();   // the next range starts where the last ended
+      for (int b : from.beg) to.beg.push_back(o + b);
+      to.h.insert(to.h.end(), from.h.begin(), from.h.end());
+      to.maxv = std::max(to.maxv, from.maxv);
+    };
+    for (const Stage& s : c->stages) {
+      if (s.type != type) continue;
+      f.procs.h.insert(f.procs.h.end(), s.procs.h.begin(), s.procs.h.end());
+      for (const LtiGroup& g : s.groups) {
+        append(f.firtaps, g.firtaps);
+        append(f.revfir, g.revfir);
+        if (!c->retain) continue;
+        append(f.col, g.col);
+        append(f.rowpair, g.rowpair);
+      }
+    }
+    if (upload_procs(c, f.procs) || upload_items(c, f.firtaps) || upload_items(c, f.revfir) || upload_items(c, f.col) ||
+        upload_items(c, f.rowpair))
+      return MG_ERR_CUDA;
+  }
+  return MG_OK;
+}
+
 // Pointers of the node table for the current structure (present processors), stage lists and launch lists.
 mg_status build_tables(mg_console* c) {
   if (c->is_graph) return build_graph_tables(c);
@@ -1197,6 +1297,7 @@ mg_status build_tables(mg_console* c) {
       if (make_stage(c, st) != MG_OK) return MG_ERR_CUDA;
       c->stages.push_back(st);
     }
+  if (join_fir_lists(c) != MG_OK) return MG_ERR_CUDA;
   // scratch pointers changed with grouping: re-upload the node table
   if (attach_dyn_maps(c) != MG_OK || upload(c, c->hpd, &c->d_procs) != MG_OK) return MG_ERR_CUDA;
   if (upload_procs(c, c->all_present) || upload_procs(c, c->all_lti_present)) return MG_ERR_CUDA;
@@ -1323,6 +1424,7 @@ mg_status build_graph_tables(mg_console* c) {
     c->gstep_stage[k] = (int)c->stages.size();
     c->stages.push_back(st);
   }
+  if (join_fir_lists(c) != MG_OK) return MG_ERR_CUDA;
   if (attach_dyn_maps(c) != MG_OK || upload(c, c->hpd, &c->d_procs) != MG_OK) return MG_ERR_CUDA;
   if (upload_procs(c, c->all_present) || upload_procs(c, c->all_lti_present)) return MG_ERR_CUDA;
   return MG_OK;
@@ -1714,6 +1816,9 @@ mg_status create_impl(mg_console* c, const mg_console_desc* d, const mg_song_des
   CK(cudaMalloc(&c->d_alphas, 4 * sizeof(float)));
   CK(cudaMalloc(&c->d_mask, std::max(1, c->P)));
   CK(cudaMalloc(&c->d_scratch_la, sizeof(float) * std::max<size_t>(1, c->songs.size())));
+  for (cudaStream_t& st : c->side) CK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+  for (cudaEvent_t* e : {&c->ev_fork, &c->ev_join[0], &c->ev_join[1]})
+    CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
   CK(cudaMalloc(&c->d_chain, sizeof(unsigned long long)));
   {
     const unsigned long long first = 1ull << 32;   // ticket 0 of generation 1 (cleared flags hold generation 0)
@@ -2016,6 +2121,10 @@ void destroy_impl(mg_console* c) {
   for (void* p : c->small_allocs) cudaFree(p);
   for (void* p : c->table_allocs) cudaFree(p);
   for (auto e : c->ev_pool) cudaEventDestroy(e);
+  for (cudaEvent_t e : {c->ev_fork, c->ev_join[0], c->ev_join[1]})
+    if (e) cudaEventDestroy(e);
+  for (cudaStream_t st : c->side)
+    if (st) cudaStreamDestroy(st);
   cudaFree(c->arena);
   cudaFree(c->scratch);
   cudaFree(c->d_params);
@@ -2518,7 +2627,7 @@ void vstage_forward(mg_console* c, const LaunchCtx& x, Stage& s) {
       break;
     default:
       for (auto& g : s.groups) {
-        run_procs(c, F_SCALE, g.procs, [&](const int* p, int n) { launch_chan_scale(x, p, n, 0); });
+        run_procs(c, F_SCALE, g.procs, [&](const int* p, int n) { launch_chan_scale(x, p, n, kScaleOfInput | kScaleOfTaps); });
         if (!c->retain) {
           run_items(c, F_COL_FWD, g.col, [&](const Item* it, int n) { launch_col_fwd_taps(x, it, n, g.col.maxv); });
           run_items(c, F_ROW_HZ, g.rowpair, [&](const Item* it, int n) { launch_row_fwd_hz(x, it, n, g.rowpair.maxv); });

@@ -227,84 +227,95 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
 // both channels of a packed transform sit at the same level up to the sampling error of the estimate; 1 for a
 // silent channel.  (Power-of-two scales, exact to apply, left the channels up to 2x apart in amplitude, and the
 // weaker channel's error moved by that factor with the estimate's rounding.)
-// which 0: the input u and the taps (in the stereo form the transforms use); 1: dL/dy.  Fixed-order sums.
+// operands: kScaleOfInput (u), kScaleOfTaps (in the stereo form the transforms use) and kScaleOfAdjoint (dL/dy) bits, one
+// CTA each.  The strided loads are latency: 1,024 threads fetch 4,096 quads (or taps) at a time, and 256 chains add
+// them in order (loading inside the chains of 256 threads, one operand after the other, took 14-20 us per launch on
+// nodes of 10 s and 42-48 on 60 s).
 __device__ __forceinline__ float unit_scale(float e) {
   if (!(e > 0.f) || !isfinite(e)) return 1.f;
   return 1.f / sqrtf(e);
 }
 
-__global__ void __launch_bounds__(256) k_chan_scale(LaunchCtx c, const int* __restrict__ procs, int which) {
-  __shared__ float red[4 * 32];
+constexpr int kScaleThreads = 1024, kScaleBatch = 4, kScaleChains = 256;
+constexpr int kScaleTile = kScaleThreads * kScaleBatch;
+__global__ void __launch_bounds__(kScaleThreads) k_chan_scale(LaunchCtx c, const int* __restrict__ procs, int operands) {
+  __shared__ float red[2 * 32];
+  __shared__ float2 tile[kScaleTile];
   const ProcDev& P = c.procs[procs[blockIdx.x]];
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  const float* x = which == 0 ? P.u : P.dy;
+  for (int i = 0; i < (int)blockIdx.y; ++i) operands &= operands - 1;
+  const int op = operands & -operands;        // this CTA's operand: the blockIdx.y-th bit
+  const float* x = op == kScaleOfInput ? P.u : P.dy;
   // self-check of the operands: a missing or misaligned signal, a row stride shorter than the signal, or missing
   // taps skip the node (its scales stay as they were) and are reported
-  if (x == nullptr || ((uintptr_t)x & 15) != 0 || P.ld < P.L || (P.ld & 3) != 0 || P.stats == nullptr ||
-      (which == 0 && P.taps == nullptr) || (which == 0 && P.type == T_D && P.aux == nullptr)) {
+  if ((op != kScaleOfTaps && (x == nullptr || ((uintptr_t)x & 15) != 0 || P.ld < P.L || (P.ld & 3) != 0)) ||
+      P.stats == nullptr || (op == kScaleOfTaps && (P.taps == nullptr || (P.type == T_D && P.aux == nullptr)))) {
     if (threadIdx.x == 0)
-      printf("k_chan_scale: node %d which %d skipped (x %p, L %d, ld %d, taps %p, stats %p)\n", procs[blockIdx.x], which,
+      printf("k_chan_scale: node %d operand %d skipped (x %p, L %d, ld %d, taps %p, stats %p)\n", procs[blockIdx.x], op,
              (const void*)x, P.L, P.ld, (const void*)P.taps, (const void*)P.stats);
     return;
   }
-  // the samples of a thread are added in order, kScaleBatch of them loaded together (the strided loads are latency:
-  // 15.3 -> 13.8 us per launch on 16 nodes of 10 s)
-  constexpr int kScaleBatch = 4;
-  const int nq = P.L >> 2;                    // whole quads of samples
-  const float4* xl = reinterpret_cast<const float4*>(x);
-  const float4* xr = reinterpret_cast<const float4*>(x + P.ld);
-  const int qs = blockDim.x * 32;             // every 32nd quad
-  for (int q0 = threadIdx.x * 32; q0 < nq; q0 += kScaleBatch * qs) {
-    float4 a[kScaleBatch], b[kScaleBatch];
+  float acc[2] = {0.f, 0.f};
+  const int t = threadIdx.x;
+  if (op != kScaleOfTaps) {
+    const int n = ((P.L >> 2) + 31) >> 5;       // every 32nd of the whole quads of samples
+    const float4* xl = reinterpret_cast<const float4*>(x);
+    const float4* xr = reinterpret_cast<const float4*>(x + P.ld);
+    for (int i0 = 0; i0 < n; i0 += kScaleTile) {
+      float4 a[kScaleBatch], b[kScaleBatch];
 #pragma unroll
-    for (int j = 0; j < kScaleBatch; ++j) {
-      const int q = min(q0 + j * qs, nq - 1);
-      a[j] = xl[q];
-      b[j] = xr[q];
-    }
-#pragma unroll
-    for (int j = 0; j < kScaleBatch; ++j)
-      if (q0 + j * qs < nq) {
-        acc[0] += a[j].x * a[j].x + a[j].y * a[j].y + a[j].z * a[j].z + a[j].w * a[j].w;
-        acc[1] += b[j].x * b[j].x + b[j].y * b[j].y + b[j].z * b[j].z + b[j].w * b[j].w;
+      for (int j = 0; j < kScaleBatch; ++j) {
+        const int i = i0 + t + j * kScaleThreads;
+        if (i < n) {
+          a[j] = xl[32 * i];
+          b[j] = xr[32 * i];
+        }
       }
-  }
-  if (which == 0 && P.type == T_D) {
-    for (int j = threadIdx.x; j < kDlyTaps * kDlyFir; j += blockDim.x) {   // c_m of both channels
-      const float a = P.aux[j], b = P.aux[kDlyTaps * kDlyFir + j];
-      acc[2] += a * a;
-      acc[3] += b * b;
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < kScaleBatch; ++j)
+        if (i0 + t + j * kScaleThreads < n)
+          tile[t + j * kScaleThreads] =
+              make_float2(a[j].x * a[j].x + a[j].y * a[j].y + a[j].z * a[j].z + a[j].w * a[j].w,
+                          b[j].x * b[j].x + b[j].y * b[j].y + b[j].z * b[j].z + b[j].w * b[j].w);
+      __syncthreads();
+      if (t < kScaleChains)
+        for (int i = t; i < min(n - i0, kScaleTile); i += kScaleChains) {
+          acc[0] += tile[i].x;
+          acc[1] += tile[i].y;
+        }
     }
-  } else if (which == 0) {
+  } else if (P.type == T_D) {
+    if (t < kScaleChains)
+      for (int j = t; j < kDlyTaps * kDlyFir; j += kScaleChains) {   // c_m of both channels
+        const float a = P.aux[j], b = P.aux[kDlyTaps * kDlyFir + j];
+        acc[0] += a * a;
+        acc[1] += b * b;
+      }
+  } else {
     const int64_t N = fft_len(P);
-    const int js = blockDim.x * 32;           // every 32nd tap
-    for (int j0 = threadIdx.x * 32; j0 < P.Nh; j0 += kScaleBatch * js) {
-      float2 t[kScaleBatch];
+    const int n = (P.Nh + 31) >> 5;             // every 32nd tap
+    for (int i0 = 0; i0 < n; i0 += kScaleTile) {
+      __syncthreads();
 #pragma unroll
-      for (int k = 0; k < kScaleBatch; ++k) {
-        const int j = min(j0 + k * js, P.Nh - 1);
-        t[k] = tap_at(P, (int64_t)j + P.n0 >= 0 ? (int64_t)j + P.n0 : N + j + P.n0, N);
+      for (int j = 0; j < kScaleBatch; ++j) {
+        const int i = i0 + t + j * kScaleThreads;
+        const int64_t at = (int64_t)32 * i + P.n0;
+        if (i < n) tile[t + j * kScaleThreads] = tap_at(P, at >= 0 ? at : N + at, N);
       }
-#pragma unroll
-      for (int k = 0; k < kScaleBatch; ++k)
-        if (j0 + k * js < P.Nh) {
-          acc[2] += t[k].x * t[k].x;
-          acc[3] += t[k].y * t[k].y;
+      __syncthreads();
+      if (t < kScaleChains)
+        for (int i = t; i < min(n - i0, kScaleTile); i += kScaleChains) {
+          acc[0] += tile[i].x * tile[i].x;
+          acc[1] += tile[i].y * tile[i].y;
         }
     }
   }
-  float out[4];
-  block_sum<4>(acc, red, out);
+  float out[2];
+  block_sum<2>(acc, red, out);
   if (threadIdx.x == 0) {
-    if (which == 0) {
-      P.stats[kScaleU] = unit_scale(out[0]);
-      P.stats[kScaleU + 1] = unit_scale(out[1]);
-      P.stats[kScaleH] = unit_scale(out[2]);
-      P.stats[kScaleH + 1] = unit_scale(out[3]);
-    } else {
-      P.stats[kScaleD] = unit_scale(out[0]);
-      P.stats[kScaleD + 1] = unit_scale(out[1]);
-    }
+    float* s = P.stats + (op == kScaleOfInput ? kScaleU : (op == kScaleOfTaps ? kScaleH : kScaleD));
+    s[0] = unit_scale(out[0]);
+    s[1] = unit_scale(out[1]);
   }
 }
 
@@ -330,8 +341,9 @@ void init_col_attributes() {
   cudaFuncSetAttribute(k_col<COL_DYBAR_KEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
 }
 
-void launch_chan_scale(const LaunchCtx& c, const int* procs, int n, int which) {
-  if (n) k_chan_scale<<<n, 256, 0, c.stream>>>(c, procs, which);
+void launch_chan_scale(const LaunchCtx& c, const int* procs, int n, int operands) {
+  const int ops = (operands & 1) + (operands >> 1 & 1) + (operands >> 2 & 1);
+  if (n) k_chan_scale<<<dim3(n, ops), kScaleThreads, 0, c.stream>>>(c, procs, operands);
 }
 void launch_col_fwd_audio(const LaunchCtx& c, const Item* items, int n, int m) { launch_col<COL_FWD_AUDIO>(c, items, n, m); }
 void launch_col_fwd_taps(const LaunchCtx& c, const Item* items, int n, int m) { launch_col<COL_FWD_TAPS>(c, items, n, m); }

@@ -201,8 +201,9 @@ void launch_col_inv_out_keep(const LaunchCtx&, const Item* items, int n, int max
 void launch_col_dybar_keep(const LaunchCtx&, const Item* items, int n, int maxN2G);
 void launch_row_bwd2(const LaunchCtx&, const Item* items, int n, int maxN1);
 void launch_col_du(const LaunchCtx&, const Item* items, int n, int maxN2G);
-// channel scales of the packed stereo transforms: which 0 = input u and taps (forward), 1 = dL/dy (backward)
-void launch_chan_scale(const LaunchCtx&, const int* procs, int n, int which);
+// channel scales of the packed stereo transforms, of one operand or of several
+constexpr int kScaleOfInput = 1, kScaleOfTaps = 2, kScaleOfAdjoint = 4;
+void launch_chan_scale(const LaunchCtx&, const int* procs, int n, int operands);
 void launch_col_dh(const LaunchCtx&, const Item* items, int n, int maxN2G);
 // reductions, loss, optimiser
 void launch_node_stats(const LaunchCtx&, const int* procs, int n, int fwd);
