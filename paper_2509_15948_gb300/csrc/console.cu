@@ -94,7 +94,8 @@ struct ItemList {
   std::vector<Item> h;
   std::vector<int> beg;  // ranges: [beg[i], beg[i+1]) for i-th proc
   Item* d = nullptr;
-  int maxv = 0;          // kernel-specific size bound (max N2*G or N1)
+  // four-step passes: ranges of the list that are launched together (end, largest size in the range; see size_classes)
+  std::vector<std::pair<int, int>> classes;
 };
 struct ProcList {
   std::vector<int> h;
@@ -662,6 +663,21 @@ void run_items(mg_console* c, int fam, const ItemList& L, F&& f) {
     if (e > b) run(c, fam, [&] { f(L.d + b, e - b); });
   }
 }
+// The same for the passes whose block size follows the transform: one launch per size class.
+template <class F>
+void run_sized(mg_console* c, int fam, const ItemList& L, F&& f) {
+  if (L.h.empty()) return;
+  for (size_t k = 0, b = 0; k < L.classes.size(); b = L.classes[k++].first) {
+    const int e = L.classes[k].first, size = L.classes[k].second;
+    if (!c->per_node) {
+      run(c, fam, [&] { f(L.d + b, e - (int)b, size); });
+      continue;
+    }
+    for (size_t i = 0; i + 1 < L.beg.size(); ++i)
+      if (L.beg[i] >= (int)b && L.beg[i] < e && L.beg[i + 1] > L.beg[i])
+        run(c, fam, [&] { f(L.d + L.beg[i], L.beg[i + 1] - L.beg[i], size); });
+  }
+}
 template <class F>
 void run_procs(mg_console* c, int fam, const ProcList& L, F&& f) {
   if (L.h.empty()) return;
@@ -736,8 +752,8 @@ void fir_synthesis(mg_console* c, const LaunchCtx& x) {
     }
     run_procs(c, F_SCALE, g.procs, [&](const int* p, int n) { launch_chan_scale(y, p, n, kScaleOfTaps); });
     if (c->retain) {
-      run_items(c, F_COL_FWD, g.col, [&](const Item* it, int n) { launch_col_fwd_taps(y, it, n, g.col.maxv); });
-      run_items(c, F_ROW_HZ, g.rowpair, [&](const Item* it, int n) { launch_row_fwd_hz(y, it, n, g.rowpair.maxv); });
+      run_sized(c, F_COL_FWD, g.col, [&](const Item* it, int n, int size) { launch_col_fwd_taps(y, it, n, size); });
+      run_sized(c, F_ROW_HZ, g.rowpair, [&](const Item* it, int n, int size) { launch_row_fwd_hz(y, it, n, size); });
     }
   }
   LtiGroup& g = c->fir[fir_slot(T_E)];
@@ -750,44 +766,44 @@ void lti_forward(mg_console* c, const LaunchCtx& x, int type, LtiGroup& g) {
   run_procs(c, F_SCALE, g.procs, [&](const int* p, int n) { launch_chan_scale(x, p, n, kScaleOfInput); });
   if (!c->retain) {   // one scratch for all stages: the filters' transforms wait for their turn
     join(c, side_of(type), c->fir_pending);
-    run_items(c, F_COL_FWD, g.col, [&](const Item* it, int n) { launch_col_fwd_taps(x, it, n, g.col.maxv); });
-    run_items(c, F_ROW_HZ, g.rowpair, [&](const Item* it, int n) { launch_row_fwd_hz(x, it, n, g.rowpair.maxv); });
+    run_sized(c, F_COL_FWD, g.col, [&](const Item* it, int n, int size) { launch_col_fwd_taps(x, it, n, size); });
+    run_sized(c, F_ROW_HZ, g.rowpair, [&](const Item* it, int n, int size) { launch_row_fwd_hz(x, it, n, size); });
   }
-  run_items(c, F_COL_FWD, g.col, [&](const Item* it, int n) { launch_col_fwd_audio(x, it, n, g.col.maxv); });
+  run_sized(c, F_COL_FWD, g.col, [&](const Item* it, int n, int size) { launch_col_fwd_audio(x, it, n, size); });
   join(c, side_of(type), c->fir_pending);
   if (c->retain) {   // U stays in T1, y_bar in T2 (natural order) for the backward
-    run_items(c, F_ROW_CONV, g.rowpair, [&](const Item* it, int n) { launch_row_conv_fwd(x, it, n, g.rowpair.maxv, true); });
-    run_items(c, F_COL_OUT, g.col, [&](const Item* it, int n) { launch_col_inv_out_keep(x, it, n, g.col.maxv); });
+    run_sized(c, F_ROW_CONV, g.rowpair, [&](const Item* it, int n, int size) { launch_row_conv_fwd(x, it, n, size, true); });
+    run_sized(c, F_COL_OUT, g.col, [&](const Item* it, int n, int size) { launch_col_inv_out_keep(x, it, n, size); });
     return;
   }
-  run_items(c, F_ROW_CONV, g.rowpair, [&](const Item* it, int n) { launch_row_conv_fwd(x, it, n, g.rowpair.maxv, false); });
-  run_items(c, F_COL_OUT, g.col, [&](const Item* it, int n) { launch_col_inv_out(x, it, n, g.col.maxv); });
+  run_sized(c, F_ROW_CONV, g.rowpair, [&](const Item* it, int n, int size) { launch_row_conv_fwd(x, it, n, size, false); });
+  run_sized(c, F_COL_OUT, g.col, [&](const Item* it, int n, int size) { launch_col_inv_out(x, it, n, size); });
 }
 
 void lti_backward(mg_console* c, const LaunchCtx& x, int type, LtiGroup& g) {
   run_procs(c, F_SCALE, g.procs, [&](const int* p, int n) { launch_chan_scale(x, p, n, kScaleOfAdjoint); });
   if (c->retain) {
-    run_items(c, F_COL_DYBAR, g.col, [&](const Item* it, int n) { launch_col_dybar_keep(x, it, n, g.col.maxv); });
+    run_sized(c, F_COL_DYBAR, g.col, [&](const Item* it, int n, int size) { launch_col_dybar_keep(x, it, n, size); });
   } else {
-    run_items(c, F_COL_FWD, g.col, [&](const Item* it, int n) { launch_col_fwd_taps(x, it, n, g.col.maxv); });
-    run_items(c, F_ROW_HZ, g.rowpair, [&](const Item* it, int n) { launch_row_fwd_hz(x, it, n, g.rowpair.maxv); });
-    run_items(c, F_COL_FWD, g.col, [&](const Item* it, int n) { launch_col_fwd_audio(x, it, n, g.col.maxv); });
-    run_items(c, F_ROW_CONV, g.rowpair, [&](const Item* it, int n) { launch_row_conv_fwd(x, it, n, g.rowpair.maxv, true); });
-    run_items(c, F_COL_DYBAR, g.col, [&](const Item* it, int n) { launch_col_dybar(x, it, n, g.col.maxv); });
+    run_sized(c, F_COL_FWD, g.col, [&](const Item* it, int n, int size) { launch_col_fwd_taps(x, it, n, size); });
+    run_sized(c, F_ROW_HZ, g.rowpair, [&](const Item* it, int n, int size) { launch_row_fwd_hz(x, it, n, size); });
+    run_sized(c, F_COL_FWD, g.col, [&](const Item* it, int n, int size) { launch_col_fwd_audio(x, it, n, size); });
+    run_sized(c, F_ROW_CONV, g.rowpair, [&](const Item* it, int n, int size) { launch_row_conv_fwd(x, it, n, size, true); });
+    run_sized(c, F_COL_DYBAR, g.col, [&](const Item* it, int n, int size) { launch_col_dybar(x, it, n, size); });
   }
-  run_items(c, F_ROW_BWD2, g.rowpair, [&](const Item* it, int n) { launch_row_bwd2(x, it, n, g.rowpair.maxv); });
+  run_sized(c, F_ROW_BWD2, g.rowpair, [&](const Item* it, int n, int size) { launch_row_bwd2(x, it, n, size); });
   // dL/dh and the FIR adjoint beside the chain; without kept spectra dL/dh reads the scratch that the next stage
   // writes, so only the adjoint leaves the console's stream
   LaunchCtx y = x;
   if (c->retain) y = fork(c, x, type, c->adj_pending);
-  run_items(c, F_COL_DH, g.col, [&](const Item* it, int n) { launch_col_dh(y, it, n, g.col.maxv); });
+  run_sized(c, F_COL_DH, g.col, [&](const Item* it, int n, int size) { launch_col_dh(y, it, n, size); });
   if (!c->retain) y = fork(c, x, type, c->adj_pending);
   if (type == T_D) run_items(c, F_FIR_ADJ, g.dlyadj, [&](const Item* it, int n) { launch_dly_adj(y, it, n); });
   if (type == T_R) {
     run_items(c, F_FIR_ADJ, g.revfir, [&](const Item* it, int n) { launch_rev_adj(y, it, n); });
     run_procs(c, F_FIR_ADJ, g.procs, [&](const int* p, int n) { launch_rev_adj_fin(y, p, n); });
   }
-  run_items(c, F_COL_DU, g.col, [&](const Item* it, int n) { launch_col_du(x, it, n, g.col.maxv); });
+  run_sized(c, F_COL_DU, g.col, [&](const Item* it, int n, int size) { launch_col_du(x, it, n, size); });
 }
 
 void stage_forward(mg_console* c, const LaunchCtx& x, Stage& s) {
@@ -1079,6 +1095,35 @@ void chain_rounds(const std::vector<int>& procs, F&& nchunks, ItemList& fwd, Ite
   if (rev) rev->beg = {0, (int)rev->h.size()};
 }
 
+// Launches of a four-step pass by size: the nodes of a list, small sizes first, are cut where the size changes, and a
+// range joins the next larger one while it is less than a wave of CTAs by itself (sizes / per threads each, 64 registers
+// a thread).  A CTA has one thread per `per` elements of the largest transform in its launch, so in one launch over
+// all sizes the smaller nodes left up to four fifths of their CTAs' threads idle at the barriers (with the column tiles'
+// own block sizes: ten songs of 5-30 s 55.2 -> 50.5 ms a step).
+constexpr int kSmCount = 152, kRegThreads = 1024;   // threads of 64 registers that an SM holds
+template <class Size, class Count>
+void size_classes(std::vector<int> nodes, int per, Size&& size, Count&& count, ItemList& L) {
+  std::stable_sort(nodes.begin(), nodes.end(), [&](int a, int b) { return size(a) < size(b); });
+  int begin = 0;
+  for (size_t k = 0; k < nodes.size(); ++k) {
+    L.beg.push_back((int)L.h.size());
+    for (int i = 0; i < count(nodes[k]); ++i) L.h.push_back(Item{nodes[k], i});
+    const int s = size(nodes[k]), end = (int)L.h.size();
+    if (k + 1 < nodes.size() && (size(nodes[k + 1]) == s || (int64_t)(end - begin) * s < (int64_t)kSmCount * kRegThreads * per))
+      continue;
+    L.classes.push_back({end, s});
+    begin = end;
+  }
+  L.beg.push_back((int)L.h.size());
+}
+
+// Column and row items of the four-step convolutions of some nodes.
+void conv_items(const std::vector<ProcDev>& dev, const std::vector<int>& nodes, ItemList& col, ItemList& row) {
+  auto n1 = [&](int v) { return dev[v].f << dev[v].logN1; };
+  size_classes(nodes, 16, [&](int v) { return dev[v].colG << dev[v].logN2; }, [&](int v) { return n1(v) / dev[v].colG; }, col);
+  size_classes(nodes, 8, n1, [&](int v) { return (1 << dev[v].logN2) / 2 + 1; }, row);
+}
+
 // Work lists of one stage (st.level, st.type, st.procs.h set): tiles or scan chunks, overlap-save blocks, or LTI
 // groups with their FFT scratch offsets (groups under the workspace limit when the spectra are not kept).
 mg_status make_stage(mg_console* c, Stage& st) {
@@ -1114,8 +1159,8 @@ mg_status make_stage(mg_console* c, Stage& st) {
     LtiGroup g;
     auto close = [&]() -> mg_status {
       if (g.procs.h.empty()) return MG_OK;
-      for (ItemList* L : {&g.col, &g.rowpair, &g.firtaps, &g.dlyadj, &g.revfir})
-        L->beg.push_back((int)L->h.size());
+      for (ItemList* L : {&g.firtaps, &g.dlyadj, &g.revfir}) L->beg.push_back((int)L->h.size());
+      conv_items(c->hpd, g.procs.h, g.col, g.rowpair);
       if (upload_procs(c, g.procs) || upload_items(c, g.col) ||
           upload_items(c, g.rowpair) || upload_items(c, g.firtaps) || upload_items(c, g.dlyadj) ||
           upload_items(c, g.revfir))
@@ -1139,13 +1184,7 @@ mg_status make_stage(mg_console* c, Stage& st) {
       d.T2 = d.T1 + N;
       d.Hz = d.T2 + N;
       g.procs.h.push_back(pi);
-      const int N1 = p.f << p.logN1, N2 = 1 << p.logN2;
-      for (ItemList* L : {&g.col, &g.rowpair, &g.firtaps, &g.dlyadj, &g.revfir})
-        L->beg.push_back((int)L->h.size());
-      for (int i = 0; i < N1 / p.colG; ++i) g.col.h.push_back(Item{pi, i});
-      g.col.maxv = std::max(g.col.maxv, N2 * p.colG);
-      for (int i = 0; i <= N2 / 2; ++i) g.rowpair.h.push_back(Item{pi, i});
-      g.rowpair.maxv = std::max(g.rowpair.maxv, N1);
+      for (ItemList* L : {&g.firtaps, &g.dlyadj, &g.revfir}) L->beg.push_back((int)L->h.size());
       if (t == T_D) {
         for (int i = 0; i < (p.Nh + 255) / 256; ++i) g.firtaps.h.push_back(Item{pi, i});
         for (int i = 0; i < 2 * kDlyTaps; ++i) g.dlyadj.h.push_back(Item{pi, i});
@@ -1170,7 +1209,6 @@ mg_status join_fir_lists(mg_console* c) {
       if (!to.beg.empty()) to.beg.pop_back();   // the next range starts where the last ended
       for (int b : from.beg) to.beg.push_back(o + b);
       to.h.insert(to.h.end(), from.h.begin(), from.h.end());
-      to.maxv = std::max(to.maxv, from.maxv);
     };
     for (const Stage& s : c->stages) {
       if (s.type != type) continue;
@@ -1178,11 +1216,9 @@ mg_status join_fir_lists(mg_console* c) {
       for (const LtiGroup& g : s.groups) {
         append(f.firtaps, g.firtaps);
         append(f.revfir, g.revfir);
-        if (!c->retain) continue;
-        append(f.col, g.col);
-        append(f.rowpair, g.rowpair);
       }
     }
+    if (c->retain && type != T_E) conv_items(c->hpd, f.procs.h, f.col, f.rowpair);
     if (upload_procs(c, f.procs) || upload_items(c, f.firtaps) || upload_items(c, f.revfir) || upload_items(c, f.col) ||
         upload_items(c, f.rowpair))
       return MG_ERR_CUDA;
@@ -2491,23 +2527,13 @@ void build_chunk(mg_console* c, const std::vector<CandPlan>& plans, const uint8_
         } else {
           LtiGroup& g = st.groups[0];
           g.procs.h.push_back(v);
-          g.col.beg.push_back((int)g.col.h.size());
-          g.rowpair.beg.push_back((int)g.rowpair.h.size());
-          const int N1 = d.f << d.logN1, N2 = 1 << d.logN2;
-          for (int i = 0; i < N1 / d.colG; ++i) g.col.h.push_back(Item{v, i});
-          for (int i = 0; i <= N2 / 2; ++i) g.rowpair.h.push_back(Item{v, i});
-          g.col.maxv = std::max(g.col.maxv, N2 * d.colG);
-          g.rowpair.maxv = std::max(g.rowpair.maxv, N1);
         }
       }
       st.elem.beg.push_back((int)st.elem.h.size());
       if ((t == T_C || t == T_N) && !c->per_node)
         chain_rounds(st.procs.h, [&](int v) { return k.vp[v].nchunks; }, st.elem, nullptr);
       st.osf.beg.push_back((int)st.osf.h.size());
-      for (auto& g : st.groups) {
-        g.col.beg.push_back((int)g.col.h.size());
-        g.rowpair.beg.push_back((int)g.rowpair.h.size());
-      }
+      for (auto& g : st.groups) conv_items(k.vp, g.procs.h, g.col, g.rowpair);
       k.stages.push_back(std::move(st));
     }
   // tables
@@ -2629,12 +2655,12 @@ void vstage_forward(mg_console* c, const LaunchCtx& x, Stage& s) {
       for (auto& g : s.groups) {
         run_procs(c, F_SCALE, g.procs, [&](const int* p, int n) { launch_chan_scale(x, p, n, kScaleOfInput | kScaleOfTaps); });
         if (!c->retain) {
-          run_items(c, F_COL_FWD, g.col, [&](const Item* it, int n) { launch_col_fwd_taps(x, it, n, g.col.maxv); });
-          run_items(c, F_ROW_HZ, g.rowpair, [&](const Item* it, int n) { launch_row_fwd_hz(x, it, n, g.rowpair.maxv); });
+          run_sized(c, F_COL_FWD, g.col, [&](const Item* it, int n, int size) { launch_col_fwd_taps(x, it, n, size); });
+          run_sized(c, F_ROW_HZ, g.rowpair, [&](const Item* it, int n, int size) { launch_row_fwd_hz(x, it, n, size); });
         }
-        run_items(c, F_COL_FWD, g.col, [&](const Item* it, int n) { launch_col_fwd_audio(x, it, n, g.col.maxv); });
-        run_items(c, F_ROW_CONV, g.rowpair, [&](const Item* it, int n) { launch_row_conv_fwd(x, it, n, g.rowpair.maxv, false); });
-        run_items(c, F_COL_OUT, g.col, [&](const Item* it, int n) { launch_col_inv_out(x, it, n, g.col.maxv); });
+        run_sized(c, F_COL_FWD, g.col, [&](const Item* it, int n, int size) { launch_col_fwd_audio(x, it, n, size); });
+        run_sized(c, F_ROW_CONV, g.rowpair, [&](const Item* it, int n, int size) { launch_row_conv_fwd(x, it, n, size, false); });
+        run_sized(c, F_COL_OUT, g.col, [&](const Item* it, int n, int size) { launch_col_inv_out(x, it, n, size); });
       }
   }
 }

@@ -28,7 +28,8 @@ constexpr int kRowThreads = 512;   // largest row block: N1 = 3072 (one thread p
 // Shared-memory layouts (padded, see mg_fftp.cuh).  Column pass: column g, row r at sm[g * col_stride + pidx(r)],
 // with col_stride = 16 (mod 16) + 16 / G so that the G columns and 16 / G rows a half-warp touches fall in
 // distinct bank pairs.  Row pass: row slot s, position k1 at sm[s * pstride(N1) + pidx(k1)].
-constexpr int kColBuf = 8192 + 512 + 160;
+constexpr int kColPad = 160;        // column buffer: the tile, its padding (1/16) and at most this for the strides
+constexpr int kColBuf = 8192 + 512 + kColPad;
 constexpr int kMaxRow = 3072;      // longest row N1 (3 x 1024)
 __host__ __device__ constexpr int col_stride(int N2, int G) { return ((N2 + (N2 >> 4) + 15) & ~15) + 16 / G; }
 
