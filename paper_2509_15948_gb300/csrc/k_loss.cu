@@ -47,9 +47,7 @@ __device__ __forceinline__ float2 chan(int c, float2 XL, float2 XR) {
 // sqrt(A_k^2 |X_c|^2 + 1e-8) of channels 0, 1 at slot pidx(k) and of channels 2, 3 at mag_slot2(k): the
 // mirror slot pidx(n - k), or for the self-mirrored bins 0 and n/2 two padding slots no element uses
 // (pidx(n) = the last slot of the padded frame, and slot 16).
-__device__ __forceinline__ int mag_slot2(int k, int n) {
-  return k == 0 ? pidx(n) : (k == (n >> 1) ? 16 : pidx(n - k));
-}
+__device__ __forceinline__ int mag_slot2(int k, int n) { return k == (n >> 1) ? 16 : pidx(n - k); }
 
 __device__ __forceinline__ float4 bin_mags(const LossRes& R, const float2* Z, int k) {
   float2 XL, XR;
@@ -129,136 +127,111 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_loss_frames(LaunchCtx c, co
       }
     }
     __syncthreads();
-    // band values from the magnitudes: with narrow bands (few Mel weights per band on average) one thread per
-    // (frame, band, channel); with wide ones one warp per (frame, band), its lanes striding the band's bins and
-    // the four channel sums reduced over the warp (a fixed xor order), so a wide high band no longer holds the
-    // whole block at the barrier behind one thread
-    // a thread only ever adds terms of one channel, so two scalars hold its sums
-    float acc0 = 0.f, acc1 = 0.f;
-    int mych = threadIdx.x & 3;
+    // Band values Y[f][b][channel] of the item into shared memory, then one pass over them for the loss terms.  The
+    // pairs (frame, band) go band by band, so that the threads of a warp run over equally long bands and read the same
+    // weights, and a weight and its bin serve all four channels.  (One thread per value, resp. one warp per pair with 20
+    // entries on average for its 32 lanes, was 60 % of the kernel's instructions.)
+    float* yv = reinterpret_cast<float*>(sm + kFrameBuf);
+    const int pairs = nb * nbands;
+    const float inv_nb = 1.f / (float)nb;   // e / nb = floor((e + 1/2) inv_nb): pairs < 2^16
+    // pair (f, b) is quad f nbands + (b + f mod 8) mod nbands: the frames of one band fall in distinct banks
+    const int rot = nbands >= 8 ? 7 : 0;
+    auto quad_of = [&](int f, int b) {
+      const int r = b + (f & rot);
+      return f * nbands + (r >= nbands ? r - nbands : r);
+    };
     if (R.band_beg[nbands] >= 16 * nbands) {
-      // a warp takes kWide (frame, band) pairs together, so that their loads and shuffles overlap; after the sums lane
-      // l finishes pair l & 7 of channel chan_of(l), and lanes 0..3 add the pairs' loss terms in pair order
-      const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5, total = nb * nbands;
-      constexpr int kWide = 4;
-      const int lch = ((lane >> 4) & 1) * 2 + ((lane >> 3) & 1);
-      for (int e0 = wid; e0 < total; e0 += kWide * nw) {
-        float y4[kWide][4];
-        int beg[kWide], len[kWide], most = 0;
-        const float2* Zf[kWide];
+      // wide bands: eight lanes per pair.  Lane l holds the sums of entries l + 8 i (mod 32), i < 4, which are then added
+      // as a warp would over its lanes with xor 16, 8, 4, 2, 1.
+      const int l8 = threadIdx.x & 7;
+      const bool h4 = l8 & 4, h2 = l8 & 2;
+      for (int e0 = threadIdx.x >> 5 << 2; e0 < pairs; e0 += blockDim.x >> 3) {
+        const int e = e0 + ((threadIdx.x >> 3) & 3);
+        const bool live = e < pairs;
+        const int bd = live ? (int)((e + 0.5f) * inv_nb) : 0, f = live ? e - bd * nb : 0;
+        const int beg = R.band_beg[bd], len = live ? R.band_beg[bd + 1] - beg : 0;
+        const int k0 = len ? R.band_bin[beg] : 0;
+        const float2* Zf = sm + f * bs;
+        float y4[4][4];
 #pragma unroll
-        for (int j = 0; j < kWide; ++j) {
-          const int e = e0 + j * nw, ee = e < total ? e : e0;
-          const int f = ee / nbands, b = ee - f * nbands;
-          Zf[j] = sm + f * bs;
-          beg[j] = R.band_beg[b];
-          len[j] = e < total ? R.band_beg[b + 1] - beg[j] : 0;
-          most = max(most, len[j]);
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int c4 = 0; c4 < 4; ++c4) y4[j][c4] = 0.f;
-        }
-        // this lane's pair and channel: its target (or earlier) value is on its way during the sums
-        const int em = e0 + (lane & 7) * nw;
-        const bool mine = (lane & 7) < kWide && em < total;
-        const size_t yi = mine ? ((size_t)t0 * nbands + em) * 4 + lch : 0;
-        const float yt = mine && mode != 0 ? Yt[yi] : 0.f;
-        for (int q = lane; q < most; q += 32) {
+          for (int ch = 0; ch < 4; ++ch) y4[i][ch] = 0.f;
+        for (int q0 = l8; q0 < len; q0 += 32) {
 #pragma unroll
-          for (int j = 0; j < kWide; ++j) {
-            if (q < len[j]) {
-              const int k = R.band_bin[beg[j] + q];
-              const float wq = R.band_w[beg[j] + q];
-              const float2 lr = Zf[j][pidx(k)], ms = Zf[j][mag_slot2(k, n)];
-              y4[j][0] = fmaf(wq, lr.x, y4[j][0]);
-              y4[j][1] = fmaf(wq, lr.y, y4[j][1]);
-              y4[j][2] = fmaf(wq, ms.x, y4[j][2]);
-              y4[j][3] = fmaf(wq, ms.y, y4[j][3]);
+          for (int i = 0; i < 4; ++i) {
+            const int q = q0 + 8 * i;
+            if (q < len) {
+              const float wq = R.band_w[beg + q];
+              const float2 lr = Zf[pidx(k0 + q)], ms = Zf[mag_slot2(k0 + q, n)];
+              y4[i][0] = fmaf(wq, lr.x, y4[i][0]);
+              y4[i][1] = fmaf(wq, lr.y, y4[i][1]);
+              y4[i][2] = fmaf(wq, ms.x, y4[i][2]);
+              y4[i][3] = fmaf(wq, ms.y, y4[i][3]);
             }
           }
         }
-        // warp sums over xor 16, 8, 4, 2, 1 (in that order for every channel): after the first step a lane keeps two
-        // channels, after the second one
-        float yh = 0.f;
+        float y[4];
 #pragma unroll
-        for (int j = 0; j < kWide; ++j) {
-          const bool h16 = lane & 16, h8 = lane & 8;
-          const float s0 = __shfl_xor_sync(0xffffffffu, h16 ? y4[j][0] : y4[j][2], 16);
-          const float s1 = __shfl_xor_sync(0xffffffffu, h16 ? y4[j][1] : y4[j][3], 16);
-          const float a0 = (h16 ? y4[j][2] : y4[j][0]) + s0, a1 = (h16 ? y4[j][3] : y4[j][1]) + s1;
-          float v = (h8 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, h8 ? a0 : a1, 8);
-          v += __shfl_xor_sync(0xffffffffu, v, 4);
-          v += __shfl_xor_sync(0xffffffffu, v, 2);
-          v += __shfl_xor_sync(0xffffffffu, v, 1);
-          if ((lane & 7) == j) yh = v;
-        }
-        float d0 = 0.f, d1 = 0.f;
-        if (mine) {
-          if (mode == 3) Yk[yi] = yh;
-          if (mode == 0) {
-            Yt[yi] = yh;
-          } else {
-            d0 = fabsf(logf(yt + kLogEps) - logf(yh + kLogEps));
-            d1 = yt - yh;
-          }
-        }
-        // lane c < 4 adds channel c of the pairs in order; the lane of pair j, channel c is 16 (c / 2) + 8 (c mod 2) + j
-#pragma unroll
-        for (int j = 0; j < kWide; ++j) {
-          const int src = (lane & 2) * 8 + (lane & 1) * 8 + j;
-          const float x0 = __shfl_sync(0xffffffffu, d0, src), x1 = __shfl_sync(0xffffffffu, d1, src);
-          const float xh = __shfl_sync(0xffffffffu, yh, src);
-          if (lane < 4 && e0 + j * nw < total) {
-            if (mode == 0) {
-              acc0 += xh * xh;
-            } else {
-              acc0 += x0;
-              acc1 += x1 * x1;
-            }
-          }
-        }
+        for (int ch = 0; ch < 4; ++ch) y[ch] = (y4[0][ch] + y4[2][ch]) + (y4[1][ch] + y4[3][ch]);
+        // after xor 4 a lane keeps two channels, after xor 2 one
+        const float s0 = __shfl_xor_sync(0xffffffffu, h4 ? y[0] : y[2], 4);
+        const float s1 = __shfl_xor_sync(0xffffffffu, h4 ? y[1] : y[3], 4);
+        const float a0 = (h4 ? y[2] : y[0]) + s0, a1 = (h4 ? y[3] : y[1]) + s1;
+        float v = (h2 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, h2 ? a0 : a1, 2);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        if (live && !(l8 & 1)) yv[4 * quad_of(f, bd) + (l8 >> 1)] = v;
       }
-      mych = lane & 3;   // lanes 0..3 hold the sums of channels 0..3, the others zeros
     } else {
-      // a thread takes kNarrow (frame, band) values of its channel together (loads in flight)
-      constexpr int kNarrow = 4;
-      const int total = nb * nbands * 4, nth = blockDim.x, ch = mych;
-      for (int e0 = threadIdx.x; e0 < total; e0 += kNarrow * nth) {
-        const float* Zf[kNarrow];
-        float yh[kNarrow], yt[kNarrow];
-        int beg[kNarrow], len[kNarrow], most = 0;
-#pragma unroll
-        for (int j = 0; j < kNarrow; ++j) {
-          const int e = e0 + j * nth, ee = e < total ? e : e0;
-          const int f = ee / (nbands * 4), b = (ee - f * (nbands * 4)) >> 2;
-          Zf[j] = reinterpret_cast<const float*>(sm + f * bs);
-          yt[j] = e < total && mode != 0 ? Yt[(size_t)t0 * nbands * 4 + e] : 0.f;
-          beg[j] = R.band_beg[b];
-          len[j] = e < total ? R.band_beg[b + 1] - beg[j] : 0;
-          most = max(most, len[j]);
-          yh[j] = 0.f;
+      for (int e = threadIdx.x; e < pairs; e += blockDim.x) {
+        const int bd = (int)((e + 0.5f) * inv_nb), f = e - bd * nb;
+        const int beg = R.band_beg[bd], len = R.band_beg[bd + 1] - beg;
+        const int k0 = len ? R.band_bin[beg] : 0;
+        const float2* Zf = sm + f * bs;
+        float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int q = 0; q < len; ++q) {
+          const float wq = R.band_w[beg + q];
+          const float2 lr = Zf[pidx(k0 + q)], ms = Zf[mag_slot2(k0 + q, n)];
+          y.x = fmaf(wq, lr.x, y.x);
+          y.y = fmaf(wq, lr.y, y.y);
+          y.z = fmaf(wq, ms.x, y.z);
+          y.w = fmaf(wq, ms.y, y.w);
         }
-        for (int q = 0; q < most; ++q) {
+        reinterpret_cast<float4*>(yv)[quad_of(f, bd)] = y;
+      }
+    }
+    __syncthreads();
+    // the values in frame order, target and kept values coalesced; a thread only ever adds terms of one channel
+    float acc0 = 0.f, acc1 = 0.f;
+    const int mych = threadIdx.x & 3;
+    {
+      const int row = nbands * 4, total = nb * row;
+      const float inv_row = 1.f / (float)row;
+      const size_t base = (size_t)t0 * row;
+      constexpr int kAhead = 4;
+      for (int e0 = threadIdx.x; e0 < total; e0 += kAhead * blockDim.x) {
+        float yt[kAhead];
+        int at[kAhead];
 #pragma unroll
-          for (int j = 0; j < kNarrow; ++j) {
-            if (q < len[j]) {
-              const int k = R.band_bin[beg[j] + q];
-              const int slot = ch < 2 ? pidx(k) : mag_slot2(k, n);
-              yh[j] = fmaf(R.band_w[beg[j] + q], Zf[j][2 * slot + (ch & 1)], yh[j]);
-            }
-          }
+        for (int j = 0; j < kAhead; ++j) {
+          const int e = e0 + j * blockDim.x, f = (int)((e + 0.5f) * inv_row);
+          const int r = e - f * row - 4 * (f & rot);
+          at[j] = f * row + (r < 0 ? r + row : r);
+          yt[j] = mode != 0 && e < total ? Yt[base + at[j]] : 0.f;
         }
 #pragma unroll
-        for (int j = 0; j < kNarrow; ++j) {
-          const int e = e0 + j * nth;
+        for (int j = 0; j < kAhead; ++j) {
+          const int e = e0 + j * blockDim.x;
           if (e >= total) continue;
-          const size_t yi = (size_t)t0 * nbands * 4 + e;
-          if (mode == 3) Yk[yi] = yh[j];
+          const float yh = yv[e];
+          if (mode == 3) Yk[base + at[j]] = yh;
           if (mode == 0) {
-            Yt[yi] = yh[j];
-            acc0 += yh[j] * yh[j];
+            Yt[base + at[j]] = yh;
+            acc0 += yh * yh;
           } else {
-            acc0 += fabsf(logf(yt[j] + kLogEps) - logf(yh[j] + kLogEps));
-            const float d = yt[j] - yh[j];
+            acc0 += fabsf(logf(yt[j] + kLogEps) - logf(yh + kLogEps));
+            const float d = yt[j] - yh;
             acc1 += d * d;
           }
         }
@@ -289,16 +262,20 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_loss_frames(LaunchCtx c, co
 #pragma unroll 4
     for (int e = threadIdx.x; e < nb * nbands * 4; e += blockDim.x) {
       const float yh = yk[e], y = yt[e];
-      const float dl = logf(yh + kLogEps) - logf(y + kLogEps);
+      // sign of the difference of the logarithms; 1e-5 apart it is the values' own (logf is good to 2e-6 here)
+      const float ph = yh + kLogEps, pt = y + kLogEps;
+      float dl = ph - pt;
+      if (!(fabsf(dl) > 1e-5f * pt)) dl = logf(ph) - logf(pt);
       const float sg = dl > 0.f ? 1.f : (dl < 0.f ? -1.f : 0.f);
-      dY[e] = c0 * sg / (yh + kLogEps) + c1 * (yh - y);
+      dY[e] = c0 * sg / ph + c1 * (yh - y);
     }
   }
   __syncthreads();
   // bins -> packed Hermitian spectrum, in place (thread owns the pair k, n - k)
   const int half = n >> 1;
+  const float inv_bins = 1.f / (float)(half + 1);   // e / (half + 1) = floor((e + 1/2) inv_bins): e < 2^14
   for (int e = threadIdx.x; e < nb * (half + 1); e += blockDim.x) {
-    const int f = e / (half + 1), k = e % (half + 1);
+    const int f = (int)((e + 0.5f) * inv_bins), k = e - f * (half + 1);
     float2* Z = sm + f * bs;
     float2 XL, XR;
     bin_spectra(Z, k, n, XL, XR);
@@ -371,7 +348,7 @@ __global__ void __launch_bounds__(256) k_loss_gather(const SongDev* __restrict__
 void launch_loss_frames(const LaunchCtx& c, const SongDev* songs, const LossRes* res, const int4* items, int n,
                         int mode, int max_dy) {
   if (!n) return;
-  const size_t smem = kFrameBuf * sizeof(float2) + (mode == 2 ? (size_t)max_dy * sizeof(float) : 0);
+  const size_t smem = kFrameBuf * sizeof(float2) + (size_t)max_dy * sizeof(float);
   switch (mode) {
     case 0: k_loss_frames<0><<<n, kLossThreads, smem, c.stream>>>(c, songs, res, items); break;
     case 1: k_loss_frames<1><<<n, kLossThreads, smem, c.stream>>>(c, songs, res, items); break;
@@ -386,12 +363,11 @@ void launch_loss_gather(const LaunchCtx& c, const SongDev* songs, const LossRes*
 }
 
 void init_loss_attributes() {
-  const int frames = kFrameBuf * sizeof(float2);
-  cudaFuncSetAttribute(k_loss_frames<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, frames);
-  cudaFuncSetAttribute(k_loss_frames<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, frames);
-  cudaFuncSetAttribute(k_loss_frames<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       frames + kLossMaxDy * (int)sizeof(float));
-  cudaFuncSetAttribute(k_loss_frames<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, frames);
+  const int most = kFrameBuf * sizeof(float2) + kLossMaxDy * (int)sizeof(float);
+  cudaFuncSetAttribute(k_loss_frames<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(k_loss_frames<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(k_loss_frames<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(k_loss_frames<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
 }  // namespace mg
