@@ -417,14 +417,15 @@ __device__ __forceinline__ float4 load_quad(const float* row, int n, int L) {
   return n < L ? tail_zero(*reinterpret_cast<const float4*>(row + n), n, L) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// Backward.  Step 1, everything that does not depend on lambda: per sample dL/dg (to aux) and the part of du
+// Backward.  Step 1, everything that does not depend on lambda: per sample dL/dg and the part of du
 // without the envelope term, the partials of dL/dT, dL/dW, dL/dR and dL/dw, and the chunk's zero-start lambda
 // aggregate.  Step 2, the chained lambda state from the right.  Step 3: lambda[n] = dL/dg[n] + alpha lambda[n+1]
 // from that state, du += 2 beta lambda m on both channels, and the partial of dL/dalpha =
 // sum lambda[n] (g[n-1] - x[n]).  With tensor maps of u and dL/dy the chunk of both arrives by TMA: step 1 reads
-// them from shared memory and leaves its part of du over dL/dy there, step 3 reads u and that part back from
-// shared memory and dL/dg from L2, and du is written once.  Without maps u and dL/dy are read from global memory
-// and step 1's part of du goes through global memory.  Both steps stream a quad at a time.
+// them from shared memory and leaves its part of du over dL/dy there and the mid signal and dL/dg over u; step 3 reads
+// all three back, and du is the only signal written (with dL/dg through global memory a sample cost 32 bytes of HBM
+// instead of 24: 16 nodes x 10 s 97 -> 82 us, 8 nodes x 60 s 256 -> 231).  Without maps u and dL/dy are read from
+// global memory, and step 1's part of du and dL/dg go through global memory.  Both steps stream a quad at a time.
 __global__ void __launch_bounds__(kThreads, 3) k_dyn_bwd(LaunchCtx c, const Item* __restrict__ items) {
   extern __shared__ unsigned char dsm[];
   float* stage = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(dsm) + 1023) & ~(uintptr_t)1023);
@@ -495,15 +496,15 @@ __global__ void __launch_bounds__(kThreads, 3) k_dyn_bwd(LaunchCtx c, const Item
         lam = fmaf(pw, dgq[e], lam);
         pw *= d.alpha;
       }
-      if (tma) {
+      if (tma) {   // a quad of every stage belongs to one thread
+        *stage_at(stage, 0, t, q) = make_float4(q_at(a, 0) + q_at(b, 0), q_at(a, 1) + q_at(b, 1),
+                                                q_at(a, 2) + q_at(b, 2), q_at(a, 3) + q_at(b, 3));
+        *stage_at(stage, 1, t, q) = make_float4(dgq[0], dgq[1], dgq[2], dgq[3]);
         *stage_at(dstage, 0, t, q) = make_float4(dl[0], dl[1], dl[2], dl[3]);
         *stage_at(dstage, 1, t, q) = make_float4(dr[0], dr[1], dr[2], dr[3]);
-      }
-      if (n < L) {
-        if (!tma) {
-          store_quad(P.du, n, L, dl[0], dl[1], dl[2], dl[3]);
-          store_quad(P.du + ld, n, L, dr[0], dr[1], dr[2], dr[3]);
-        }
+      } else if (n < L) {
+        store_quad(P.du, n, L, dl[0], dl[1], dl[2], dl[3]);
+        store_quad(P.du + ld, n, L, dr[0], dr[1], dr[2], dr[3]);
         store_quad(P.aux, n, L, dgq[0], dgq[1], dgq[2], dgq[3]);
       }
     }
@@ -526,13 +527,18 @@ __global__ void __launch_bounds__(kThreads, 3) k_dyn_bwd(LaunchCtx c, const Item
   float s = 0.f;
 #pragma unroll
   for (int q = 0; q < kPer / 4; ++q) {
-    const float4 a = uq(0, q), b = uq(1, q);
+    const float4 a = tma ? stage_quad(stage, 0, t, q) : load_quad(P.u, n0 + 4 * q, L);
+    const float4 b = tma ? make_float4(0.f, 0.f, 0.f, 0.f) : load_quad(P.u + ld, n0 + 4 * q, L);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      m[4 * q + e] = q_at(a, e) + q_at(b, e);
+      m[4 * q + e] = tma ? q_at(a, e) : q_at(a, e) + q_at(b, e);
       s = d.alpha * s + d.beta * (m[4 * q + e] * m[4 * q + e]);
     }
   }
+  auto dg_quad = [&](int q) {
+    const int n = n0 + 4 * q;
+    return tma ? mask_quad(stage_quad(stage, 1, t, q), n, L) : load_quad(P.aux, n, L);
+  };
   float g = scan_fwd_excl(s, dec, dec + 32, P.carry[it.idx], sm);
 #pragma unroll
   for (int j = 0; j < kPer; ++j) {
@@ -543,7 +549,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_dyn_bwd(LaunchCtx c, const Item
   float rl = 0.f;
 #pragma unroll
   for (int q = kPer / 4 - 1; q >= 0; --q) {
-    const float4 dg = load_quad(P.aux, n0 + 4 * q, L);
+    const float4 dg = dg_quad(q);
 #pragma unroll
     for (int e = 3; e >= 0; --e) rl = q_at(dg, e) + d.alpha * rl;
   }
@@ -552,7 +558,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_dyn_bwd(LaunchCtx c, const Item
 #pragma unroll
   for (int q = kPer / 4 - 1; q >= 0; --q) {
     const int n = n0 + 4 * q;
-    const float4 dg = load_quad(P.aux, n, L);
+    const float4 dg = dg_quad(q);
     const float4 a = tma ? stage_quad(dstage, 0, t, q) : load_quad(P.du, n, L);
     const float4 b = tma ? stage_quad(dstage, 1, t, q) : load_quad(P.du + ld, n, L);
     float dl[4] = {a.x, a.y, a.z, a.w}, dr[4] = {b.x, b.y, b.z, b.w};
