@@ -101,27 +101,32 @@ __global__ void __launch_bounds__(256) k_gs_bwd(LaunchCtx c, const Item* __restr
   }
 }
 
-// Eq. (3) sums: out[s] = sum over its inputs (mix node m and output node o).
+// Eq. (3) sums: out[s] = sum over its inputs (mix node m and output node o), in input order.  A thread makes one quad of
+// one channel (blockIdx.y: channel and 1,024-sample part of the tile) with the loads of eight inputs together: with
+// four quads of both channels per thread, one input after the other, the output sum of 5 chains x 10 s took 16 us on 108
+// CTAs; now 8 (24 tracks x 30 s are at HBM rate either way, 52 us).
 __global__ void __launch_bounds__(256) k_sum(float* const* outs, const float* const* ins, const int* in_beg,
                                              const int* Ls, const int* lds, const Item* items, int tile) {
   const Item it = items[blockIdx.x];
   const int s = it.proc, L = Ls[s], ld = lds[s];
   const int beg = in_beg[s], end = in_beg[s + 1];
-  const int v0 = it.idx * (tile / 4);
-  const int vend = min(v0 + tile / 4, (L + 3) >> 2);
-  float4* ol = reinterpret_cast<float4*>(outs[s]);
-  float4* orr = reinterpret_cast<float4*>(outs[s] + ld);
-  for (int v = v0 + threadIdx.x; v < vend; v += blockDim.x) {
-    float4 al = make_float4(0.f, 0.f, 0.f, 0.f), ar = al;
-    for (int j = beg; j < end; ++j) {
-      const float4 a = reinterpret_cast<const float4*>(ins[j])[v];
-      const float4 b = reinterpret_cast<const float4*>(ins[j] + ld)[v];
-      al.x += a.x; al.y += a.y; al.z += a.z; al.w += a.w;
-      ar.x += b.x; ar.y += b.y; ar.z += b.z; ar.w += b.w;
-    }
-    ol[v] = al;
-    orr[v] = ar;
+  const int v = it.idx * (tile / 4) + (blockIdx.y >> 1) * 256 + threadIdx.x;
+  if (v >= (L + 3) >> 2) return;
+  const int64_t o = (int64_t)(blockIdx.y & 1) * ld;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  constexpr int kAhead = 8;
+  for (int j0 = beg; j0 < end; j0 += kAhead) {
+    float4 a[kAhead];
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j)
+      if (j0 + j < end) a[j] = reinterpret_cast<const float4*>(ins[j0 + j] + o)[v];
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j)
+      if (j0 + j < end) {
+        acc.x += a[j].x; acc.y += a[j].y; acc.z += a[j].z; acc.w += a[j].w;
+      }
   }
+  reinterpret_cast<float4*>(outs[s] + o)[v] = acc;
 }
 
 __global__ void k_ingest(const float* __restrict__ mono, float* __restrict__ st, int L, int ld) {
@@ -144,13 +149,28 @@ __global__ void k_ingest_song(const float* __restrict__ mono, float* const* __re
   }
 }
 
-__global__ void k_copy_mix(const SongDev* songs, int nsongs, float* out, const int64_t* offs) {
+// Mixes to the caller's rows, which may start at any sample: four samples of both channels of a thread in flight.
+constexpr int kCopyPer = 4;
+__global__ void __launch_bounds__(256) k_copy_mix(const SongDev* songs, int nsongs, float* out, const int64_t* offs) {
   const int s = blockIdx.y;
   const SongDev& S = songs[s];
+  const int L = S.L, ld = S.ld, step = gridDim.x * blockDim.x;
+  const float* mix = S.mix;
   float* o = out + offs[s];
-  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < S.L; n += gridDim.x * blockDim.x) {
-    o[n] = S.mix[n];
-    o[S.L + n] = S.mix[S.ld + n];
+  for (int n0 = blockIdx.x * blockDim.x + threadIdx.x; n0 < L; n0 += kCopyPer * step) {
+    float a[kCopyPer], b[kCopyPer];
+#pragma unroll
+    for (int j = 0; j < kCopyPer; ++j)
+      if (n0 + (int64_t)j * step < L) {
+        a[j] = mix[n0 + j * step];
+        b[j] = mix[ld + n0 + j * step];
+      }
+#pragma unroll
+    for (int j = 0; j < kCopyPer; ++j)
+      if (n0 + (int64_t)j * step < L) {
+        o[n0 + j * step] = a[j];
+        o[L + n0 + j * step] = b[j];
+      }
   }
 }
 
@@ -162,7 +182,7 @@ void launch_gs_bwd(const LaunchCtx& c, const Item* items, int n) {
 }
 void launch_sum(cudaStream_t st, float* const* outs, const float* const* ins, const int* in_beg, const int* L,
                 const int* ld, const Item* items, int n, int tile) {
-  if (n) k_sum<<<n, 256, 0, st>>>(outs, ins, in_beg, L, ld, items, tile);
+  if (n) k_sum<<<dim3(n, 2 * (tile / 1024)), 256, 0, st>>>(outs, ins, in_beg, L, ld, items, tile);   // tile: 1,024 m
 }
 void launch_ingest(cudaStream_t st, const float* mono, float* stereo, int L, int ld) {
   k_ingest<<<min(1024, (L + 255) / 256), 256, 0, st>>>(mono, stereo, L, ld);

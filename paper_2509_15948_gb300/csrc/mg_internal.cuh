@@ -30,7 +30,7 @@ constexpr int kRevFG = 16;                 // frames per reverb work item
 constexpr int kDynChunk = 4096;            // samples per envelope-scan work item (256 threads x 16)
 constexpr int kElemTile = 4096;            // samples per elementwise work item (default; tuned per console)
 constexpr int kElemTileMin = 1024;         // smallest candidate of the packing tuner
-constexpr int kGatherTile = 1024;          // samples per work item of the loss adjoint's overlap-add
+constexpr int kGatherTile = 256;           // samples per work item of the loss adjoint's overlap-add
 constexpr int kLossPerDiv = 4;             // loss work items hold 8192 / n_fft frames, or down to a quarter of that
 constexpr float kEnvEps = 1e-8f;           // G_u = ln(g + eps)
 constexpr int kLossFrameBuf = 8192 + 512 + 128;   // padded frames of one loss work item (float2)
