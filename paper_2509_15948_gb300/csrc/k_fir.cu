@@ -17,34 +17,63 @@ __device__ __forceinline__ float softplusf_(float x) { return x > 20.f ? x : log
 // equalizer
 // ------------------------------------------------------------------------------------------------
 // Both sums are serial chains of 1,023 dependent multiply-adds whose indices walk a 2,047-entry cosine table, so what
-// bounds them is latency: kEqParts CTAs per node, one output per thread (the taps at +n and -n share a sum).  With one
-// CTA per node and eight, resp. four, outputs per thread in turn they took 121 and 66 us per launch for any batch up to
-// a node per SM; now 22 and 23.
+// bounds them is latency: kEqParts CTAs per node, one output per thread (the taps at +n and -n share a sum), and eight
+// table positions at a time from one, so that the walk is not a second chain beside the sum.  With one CTA per node and
+// eight, resp. four, outputs per thread in turn they took 121 and 66 us per launch for any batch up to a node per SM; with
+// one output per thread and the walk step by step 22 and 23; now 15 and 16.
 constexpr int kEqParts = 8, kEqFirThreads = kEqParams / kEqParts;
+constexpr int kEqPad = 7;   // term k of a sum sits at k + kEqPad: eight terms from k = 1, 9, ... on are two aligned float4
+
+// acc + sum_{k=1}^{1023} coef[k + kEqPad] cs[k step mod 2047], in order (step < 2047)
+__device__ __forceinline__ float eq_cos_sum(const float* coef, const float* cs, unsigned step, float acc) {
+  constexpr unsigned N = kEqTaps;
+  auto wrap = [](unsigned x) { return min(x, x - N); };   // x mod N for x < 2 N
+  unsigned off[8];
+  off[0] = 0;
+#pragma unroll
+  for (int j = 1; j < 8; ++j) off[j] = wrap(off[j - 1] + step);
+  const unsigned step8 = wrap(off[7] + step);
+  unsigned base = step;
+#pragma unroll 2
+  for (int k = 1; k + 8 <= kEqParams; k += 8) {
+    const float4 a = *reinterpret_cast<const float4*>(coef + k + kEqPad);
+    const float4 b = *reinterpret_cast<const float4*>(coef + k + kEqPad + 4);
+    float x[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) x[j] = cs[wrap(base + off[j])];
+    base = wrap(base + step8);
+    acc = fmaf(a.x, x[0], acc);
+    acc = fmaf(a.y, x[1], acc);
+    acc = fmaf(a.z, x[2], acc);
+    acc = fmaf(a.w, x[3], acc);
+    acc = fmaf(b.x, x[4], acc);
+    acc = fmaf(b.y, x[5], acc);
+    acc = fmaf(b.z, x[6], acc);
+    acc = fmaf(b.w, x[7], acc);
+  }
+#pragma unroll
+  for (int j = 0; j < 7; ++j) acc = fmaf(coef[kEqParams - 7 + j + kEqPad], cs[wrap(base + off[j])], acc);
+  return acc;
+}
+static_assert((kEqParams - 1) % 8 == 7 && kEqHalf == kEqParams - 1, "eq_cos_sum takes groups of eight and seven more");
+
 __global__ void __launch_bounds__(kEqFirThreads) k_eq_fir(LaunchCtx c, const int* __restrict__ procs) {
-  __shared__ float ep[kEqParams];
+  __shared__ __align__(16) float ep[kEqParams + kEqPad + 1];
   __shared__ float cs[kEqTaps];
   const ProcDev& P = c.procs[procs[blockIdx.x]];
-  for (int k = threadIdx.x; k < kEqParams; k += blockDim.x) ep[k] = expf(P.p[k]);
+  for (int k = threadIdx.x; k < kEqParams; k += blockDim.x) ep[k + kEqPad] = expf(P.p[k]);
   for (int m = threadIdx.x; m < kEqTaps; m += blockDim.x) cs[m] = c.tab.cos_eq[m];
   __syncthreads();
   const int an = blockIdx.y * kEqFirThreads + threadIdx.x;   // |n|
-  float acc = 0.f;
-  int idx = 0;
-#pragma unroll 8
-  for (int k = 1; k < kEqParams; ++k) {
-    idx += an;
-    if (idx >= kEqTaps) idx -= kEqTaps;
-    acc = fmaf(ep[k], cs[idx], acc);
-  }
+  const float acc = eq_cos_sum(ep, cs, an, 0.f), e0 = ep[kEqPad];
   const int jp = kEqHalf + an, jm = kEqHalf - an;
-  P.taps[jp] = c.tab.hann_eq[jp] * (ep[0] + 2.f * acc) * (1.f / kEqTaps);
-  P.taps[jm] = c.tab.hann_eq[jm] * (ep[0] + 2.f * acc) * (1.f / kEqTaps);
+  P.taps[jp] = c.tab.hann_eq[jp] * (e0 + 2.f * acc) * (1.f / kEqTaps);
+  P.taps[jm] = c.tab.hann_eq[jm] * (e0 + 2.f * acc) * (1.f / kEqTaps);
 }
 
 // dL/dp_k = e^{p_k} (c_k / N) sum_n dh[n] v[n] cos(2 pi k n / N), c_0 = 1, c_k = 2; dh = dh_l + dh_r.
 __global__ void __launch_bounds__(kEqFirThreads) k_eq_fir_adj(LaunchCtx c, const int* __restrict__ procs) {
-  __shared__ float e[kEqParams];
+  __shared__ __align__(16) float e[kEqParams + kEqPad + 1];
   __shared__ float cs[kEqTaps];
   const ProcDev& P = c.procs[procs[blockIdx.x]];
   for (int m = threadIdx.x; m < kEqTaps; m += blockDim.x) cs[m] = c.tab.cos_eq[m];
@@ -52,18 +81,11 @@ __global__ void __launch_bounds__(kEqFirThreads) k_eq_fir_adj(LaunchCtx c, const
     const int jp = kEqHalf + m, jm = kEqHalf - m;
     const float dp = (P.dtaps[jp] + P.dtaps[P.Nh + jp]) * c.tab.hann_eq[jp];
     const float dm = (P.dtaps[jm] + P.dtaps[P.Nh + jm]) * c.tab.hann_eq[jm];
-    e[m] = m == 0 ? dp : dp + dm;
+    e[m + kEqPad] = m == 0 ? dp : dp + dm;
   }
   __syncthreads();
   const int k = blockIdx.y * kEqFirThreads + threadIdx.x;
-  float acc = e[0];
-  int idx = 0;
-#pragma unroll 8
-  for (int m = 1; m <= kEqHalf; ++m) {
-    idx += k;
-    if (idx >= kEqTaps) idx -= kEqTaps;
-    acc = fmaf(e[m], cs[idx], acc);
-  }
+  const float acc = eq_cos_sum(e, cs, k, e[kEqPad]);
   P.gp[k] = expf(P.p[k]) * (k == 0 ? 1.f : 2.f) * (1.f / kEqTaps) * acc;
 }
 
