@@ -6,18 +6,6 @@
 
 namespace mg {
 
-// Sum of a double over the block (blockDim.x a multiple of 32, at most 512) in a fixed order; every thread gets it.
-__device__ __forceinline__ double block_total(double v, double* red /* >= 16 */) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double s = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-  return s;
-}
-
 // One CTA per processor: stats[0..1] = sums of the forward partials (LTI: E_ybar_mid, E_u_mid); stats[4..11] = sums
 // of the backward partials.  The rows (one per work item, up to about a thousand) are latency: 16 row groups of 8
 // columns read them side by side (with one group the kernel took 6-50 us per launch, waiting for one load after
@@ -51,23 +39,56 @@ __global__ void __launch_bounds__(kStatThreads) k_node_stats(LaunchCtx c, const 
 // Latency-bound: a warp per (resolution, sum) adds the work items' partials, a thread per (resolution, set) forms the
 // loss terms, a thread per processor its regularisers.  (One thread going through items, terms and processors in turn
 // took 134 us on a song of 5 chains, 476 us on 20 and 748 us on 40: double-precision logarithms and dependent loads.)
-constexpr int kFinThreads = 256;
+// The sums (18 warps) and the processors (the other 14) run side by side, and only the threads whose result counts
+// touch double precision, of which an SM does two operations per cycle: 21 -> 16 us on a song of 30 chains.
+constexpr int kFinThreads = 1024, kFinSumWarps = 18, kFinRegWarps = kFinThreads / 32 - kFinSumWarps;
 __global__ void __launch_bounds__(kFinThreads) k_loss_finalize(LaunchCtx c, const SongDev* __restrict__ songs,
                                                                const LossRes* __restrict__ resv, int nres,
                                                                const float* __restrict__ alphas, int mode,
                                                                float* out_losses, float* out_la, int la_stride) {
-  __shared__ double sums[3][6], term[3][3], red[16];
+  __shared__ double sums[3][6], term[3][3], reg[kFinRegWarps][2];
   const int si = blockIdx.x;
   const SongDev& S = songs[si];
   const int t = threadIdx.x, lane = t & 31;
-  for (int p = t >> 5; p < nres * 6; p += kFinThreads / 32) {
-    const int r = p / 6, j = p % 6;
-    double s = 0.0;
+  if (t >> 5 < kFinSumWarps) {
+    const int p = t >> 5, r = p / 6, j = p % 6;
+    if (r < nres) {
+      double s = 0.0;
 #pragma unroll 4
-    for (int i = lane; i < S.litems[r]; i += 32) s += (double)S.lpart[((size_t)r * S.lcap + i) * 6 + j];
+      for (int i = lane; i < S.litems[r]; i += 32) s += (double)S.lpart[((size_t)r * S.lcap + i) * 6 + j];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) sums[r][j] = s;
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) sums[r][j] = s;
+    }
+  } else if (mode == 1) {
+    constexpr int kFirst = kFinSumWarps * 32;
+    double lg = 0.0, lp = 0.0;
+    for (int i = S.pbeg + t - kFirst; i < S.pend; i += kFinThreads - kFirst) {
+      const ProcDev& P = c.procs[i];
+      if (!P.present) continue;
+      double w = 1.0 / (1.0 + exp(-(double)c.q[P.qidx]));
+      if (c.mask) w *= (double)c.mask[P.qidx];
+      lp += w;
+      if (P.type == T_E || P.type == T_R || P.type == T_D) {
+        const double ey = P.stats[0], eu = P.stats[1];
+        const double d = 0.5 * log(ey + 1e-12) - 0.5 * log(eu + 1e-12);
+        lg += fabs(d);
+        const double sg = d > 0.0 ? 1.0 : (d < 0.0 ? -1.0 : 0.0);
+        P.stats[2] = (float)(c.alpha_g * sg / (ey + 1e-12));
+        P.stats[3] = (float)(-c.alpha_g * sg / (eu + 1e-12));
+      }
+    }
+    if (S.pbeg + (t & ~31) - kFirst < S.pend) {   // the warp has a processor
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        lg += __shfl_xor_sync(0xffffffffu, lg, o);
+        lp += __shfl_xor_sync(0xffffffffu, lp, o);
+      }
+    }
+    if (lane == 0) {
+      reg[(t >> 5) - kFinSumWarps][0] = lg;
+      reg[(t >> 5) - kFinSumWarps][1] = lp;
+    }
   }
   __syncthreads();
   if (mode == 0) {
@@ -92,32 +113,22 @@ __global__ void __launch_bounds__(kFinThreads) k_loss_finalize(LaunchCtx c, cons
     S.coef[r * 6 + 2 * k + 1] = c1;
   }
   __syncthreads();
+  if (t != 0) return;
   double Lset[3] = {0.0, 0.0, 0.0};
   for (int r = 0; r < nres; ++r)
     for (int k = 0; k < 3; ++k) Lset[k] += term[r][k];
   const double La = alphas[0] * Lset[0] + alphas[1] * Lset[1] + alphas[2] * Lset[2];
   if (mode == 2) {
-    if (t == 0) out_la[si * la_stride] = (float)La;
+    out_la[si * la_stride] = (float)La;
     return;
   }
-  double lg = 0.0, lp = 0.0;
-  for (int i = S.pbeg + t; i < S.pend; i += kFinThreads) {
-    const ProcDev& P = c.procs[i];
-    if (!P.present) continue;
-    double w = 1.0 / (1.0 + exp(-(double)c.q[P.qidx]));
-    if (c.mask) w *= (double)c.mask[P.qidx];
-    lp += w;
-    if (P.type == T_E || P.type == T_R || P.type == T_D) {
-      const double ey = P.stats[0], eu = P.stats[1];
-      const double d = 0.5 * log(ey + 1e-12) - 0.5 * log(eu + 1e-12);
-      lg += fabs(d);
-      const double sg = d > 0.0 ? 1.0 : (d < 0.0 ? -1.0 : 0.0);
-      P.stats[2] = (float)(c.alpha_g * sg / (ey + 1e-12));
-      P.stats[3] = (float)(-c.alpha_g * sg / (eu + 1e-12));
+  if (out_losses) {
+    double Lg = 0.0, Lp = 0.0;
+    const int warps = min(kFinRegWarps, (S.pend - S.pbeg + 31) / 32);
+    for (int w = 0; w < warps; ++w) {
+      Lg += reg[w][0];
+      Lp += reg[w][1];
     }
-  }
-  const double Lg = block_total(lg, red), Lp = block_total(lp, red);
-  if (t == 0 && out_losses) {
     const double ap = c.hyper[0];
     float* o = out_losses + si * 7;
     o[0] = (float)La;
