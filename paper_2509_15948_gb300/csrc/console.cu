@@ -119,7 +119,8 @@ struct GNode {
 struct Stage {
   int level, type;
   ProcList procs;
-  ItemList elem;                 // g, s, c, n (tile / chunk items)
+  ItemList elem;                 // g, s, c, n (tile / chunk items); g and s: those without a partner
+  ItemList pair;                 // s: tile items of the imagers with a gain/pan right after them, which run as one pass
   ItemList elem_rev;             // c, n: chunk items in reverse order per node (the chained backward)
   ItemList chain_f, chain_b;     // c, n: the same chunks in rounds across nodes (batched launches)
   ItemList osf;                  // e: overlap-save blocks
@@ -811,6 +812,7 @@ void stage_forward(mg_console* c, const LaunchCtx& x, Stage& s) {
   switch (s.type) {
     case T_G:
     case T_S:
+      run_items(c, F_GS_FWD, s.pair, [&](const Item* it, int n) { launch_sg_fwd(x, it, n); });
       run_items(c, F_GS_FWD, s.elem, [&](const Item* it, int n) { launch_gs_fwd(x, it, n); });
       break;
     case T_C:
@@ -830,6 +832,7 @@ void stage_backward(mg_console* c, const LaunchCtx& x, Stage& s) {
   switch (s.type) {
     case T_G:
     case T_S:
+      run_items(c, F_GS_BWD, s.pair, [&](const Item* it, int n) { launch_sg_bwd(x, it, n); });
       run_items(c, F_GS_BWD, s.elem, [&](const Item* it, int n) { launch_gs_bwd(x, it, n); });
       break;
     case T_C:
@@ -1135,6 +1138,12 @@ mg_status make_stage(mg_console* c, Stage& st) {
   const int64_t limit = c->desc.workspace_limit_bytes > 0 ? c->desc.workspace_limit_bytes : INT64_MAX;
   if (t == T_G || t == T_S || t == T_C || t == T_N) {
     for (int pi : st.procs.h) {
+      const bool paired = (t == T_G || t == T_S) && c->hpd[pi].pair >= 0;
+      if (paired) {
+        st.pair.beg.push_back((int)st.pair.h.size());
+        for (int i = 0; t == T_S && i < c->procs[pi].nbrows; ++i) st.pair.h.push_back(Item{pi, i});
+        continue;
+      }
       st.elem.beg.push_back((int)st.elem.h.size());
       st.elem_rev.beg.push_back((int)st.elem_rev.h.size());
       const int nt = (t == T_C || t == T_N) ? c->procs[pi].nchunks : c->procs[pi].nbrows;
@@ -1142,11 +1151,12 @@ mg_status make_stage(mg_console* c, Stage& st) {
       if (t == T_C || t == T_N)
         for (int i = nt - 1; i >= 0; --i) st.elem_rev.h.push_back(Item{pi, i});
     }
+    st.pair.beg.push_back((int)st.pair.h.size());
     st.elem.beg.push_back((int)st.elem.h.size());
     st.elem_rev.beg.push_back((int)st.elem_rev.h.size());
     if (t == T_C || t == T_N)
       chain_rounds(st.procs.h, [&](int pi) { return c->procs[pi].nchunks; }, st.chain_f, &st.chain_b);
-    if (upload_items(c, st.elem) || upload_items(c, st.elem_rev) || upload_items(c, st.chain_f) ||
+    if (upload_items(c, st.pair) || upload_items(c, st.elem) || upload_items(c, st.elem_rev) || upload_items(c, st.chain_f) ||
         upload_items(c, st.chain_b) || upload_procs(c, st.procs))
       return MG_ERR_CUDA;
   } else if (t == T_E) {
@@ -1240,6 +1250,7 @@ mg_status build_tables(mg_console* c) {
   for (size_t ci = 0; ci < c->chains.size(); ++ci) {
     const HostChain& ch = c->chains[ci];
     size_t cur = ch.o_in;
+    int last = -1;
     for (int pi : ch.procs) {
       HostProc& p = c->procs[pi];
       ProcDev& d = c->hpd[pi];
@@ -1248,6 +1259,11 @@ mg_status build_tables(mg_console* c) {
       d.u = (const float*)A(cur);
       d.y = (float*)A(p.o_y);
       cur = p.o_y;
+      if (p.type == T_G && last >= 0 && c->procs[last].type == T_S) {
+        d.pair = last;
+        c->hpd[last].pair = pi;
+      }
+      last = pi;
     }
     chain_out[ci] = cur;
   }
@@ -1271,6 +1287,7 @@ mg_status build_tables(mg_console* c) {
         d.dy = (const float*)A(cur);
         const size_t nxt = useA ? ch.o_dA : ch.o_dB;
         d.du = (float*)A(nxt);
+        if (c->procs[pi].type == T_G && d.pair >= 0) continue;   // the imager before it writes the pair's adjoint
         cur = nxt;
         useA = !useA;
       }
@@ -3287,8 +3304,17 @@ mg_status mg_debug_read(const mg_console* cc, int32_t proc, int32_t what, float*
   if (!src) return fail(c, MG_ERR_INVALID, "buffer not present for this processor");
   if (n != rows * cols) return fail(c, MG_ERR_INVALID, "size mismatch");
   CK(cudaStreamSynchronize(c->stream));
+  // between an imager and the gain/pan after it the adjoint is not stored: the gain/pan's dL/dy times its two gains
+  const bool between = d.pair >= 0 && ((what == 3 && p.type == T_G) || (what == 5 && p.type == T_S));
+  const ProcDev& g = p.type == T_G || !between ? d : c->hpd[d.pair];
+  if (between) src = g.dy;
   CK(cudaMemcpy2D(host_out, cols * sizeof(float), src, ld * sizeof(float), cols * sizeof(float), rows,
                   cudaMemcpyDeviceToHost));
+  if (between) {
+    float k[2];
+    CK(cudaMemcpy(k, g.stats + kStatPairGain, sizeof(k), cudaMemcpyDeviceToHost));
+    for (int64_t i = 0; i < 2 * cols; ++i) host_out[i] *= k[i >= cols];
+  }
   return MG_OK;
 }
 

@@ -15,6 +15,7 @@ constexpr int kNPart = 8;                  // partial sums per work item
 // the packed stereo transforms (u, taps, dL/dy_bar; left then right)
 constexpr int kStatsFloats = 32;
 constexpr int kScaleU = 16, kScaleH = 18, kScaleD = 20;
+constexpr int kStatPairGain = 24;          // gain/pan of a pair: dL/du = this (left, right) times dL/dy
 constexpr int kEqTaps = 2047;              // Sec. 3.3
 constexpr int kEqHalf = 1023;
 constexpr int kEqParams = 1024;
@@ -52,6 +53,7 @@ struct ProcDev {
   int type, song, qidx, L, ld;             // ld: channel stride of every [2][ld] buffer
   int present;                             // 0 once removed by structural pruning
   int rev;                                 // rank among reverbs (noise index), -1 otherwise
+  int pair = -1;                           // imager with a gain/pan right after it (and the reverse): the other's index
   const float* u;                          // forward input  [2][ld]
   float* y;                                // forward output [2][ld]
   const float* dy;                         // adjoint of y
@@ -159,6 +161,9 @@ struct LaunchCtx {
 // elementwise processors, sums, ingest
 void launch_gs_fwd(const LaunchCtx&, const Item* items, int n);
 void launch_gs_bwd(const LaunchCtx&, const Item* items, int n);
+// an imager (the items' processors) and the gain/pan after it in one pass
+void launch_sg_fwd(const LaunchCtx&, const Item* items, int n);
+void launch_sg_bwd(const LaunchCtx&, const Item* items, int n);
 void launch_sum(cudaStream_t, float* const* outs, const float* const* ins, const int* in_beg, const int* L,
                 const int* ld, const Item* items, int n, int tile);
 void launch_ingest(cudaStream_t, const float* mono, float* stereo, int L, int ld);
