@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
   const ProcDev& P = c.procs[it.proc];
   const int G = P.colG, logG = __ffs(G) - 1;
   const int logN2 = P.logN2, N2 = 1 << logN2, N1 = rows_len(P);
-  const int64_t N = fft_len(P);
+  const int N = fft_len(P);
   const int cs = col_stride(N2, G);
   constexpr bool kOut = MODE == COL_INV_OUT || MODE == COL_INV_OUT_KEEP;
   constexpr bool kDybar = MODE == COL_DYBAR || MODE == COL_DYBAR_KEEP;
@@ -54,12 +54,12 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
   const int g = threadIdx.x & (G - 1), r0 = threadIdx.x >> logG;
   const int RS = blockDim.x >> logG;
   const int n1 = it.idx * G + g;
-  const int64_t nbase = (int64_t)n1 + (int64_t)r0 * N1;
-  const int64_t nstep = (int64_t)RS * N1;
+  const int nbase = n1 + r0 * N1;
+  const int nstep = RS * N1;
   float2* col = sm + g * cs;
   auto row_of = [&](int s) { return r0 + s * RS; };
   auto live = [&](int s) { return row_of(s) < N2; };
-  auto pos = [&](int s) { return nbase + (int64_t)s * nstep; };
+  auto pos = [&](int s) { return nbase + s * nstep; };
 
   // The column transforms run with the batch-fastest thread order (eight adjacent columns of one row per
   // quarter warp), so their first pass reads, and a forward transform's last pass writes, global memory
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
   auto tw_store = [&](float2* dst) {
     return [&, dst](int gg, int k2, float2 v) {
       const float2* t = ctw + gg * kColTwS;
-      dst[n1b + gg + (int64_t)N1 * k2] = cmul(v, cmul(t[k2 & 63], t[64 + (k2 >> 6)]));
+      dst[n1b + gg + N1 * k2] = cmul(v, cmul(t[k2 & 63], t[64 + (k2 >> 6)]));
     };
   };
 
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
     const int L = P.L, ld = P.ld;
     const float2 sc = chan_scale(P, MODE == COL_FWD_AUDIO ? kScaleU : kScaleH);
     fft_p_io<false, 1, true>(sm, logN2, G, cs, c.tab.ptw, [&](int gg, int n2) {
-      const int64_t n = n1b + gg + (int64_t)N1 * n2;
+      const int n = n1b + gg + N1 * n2;
       if (MODE == COL_FWD_AUDIO) return n < L ? make_float2(u[n] * sc.x, u[ld + n] * sc.y) : make_float2(0.f, 0.f);
       const float2 t = tap_at(P, n, N);
       return make_float2(t.x * sc.x, t.y * sc.y);
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
   if (MODE != COL_DYBAR_KEEP) {
     const float2* src = (MODE == COL_INV_OUT || MODE == COL_DH) ? P.T1 : P.T2;
     fft_p_io<true, 1, true>(sm, logN2, G, cs, c.tab.ptw,
-                            [&](int gg, int n2) { return src[n1b + gg + (int64_t)N1 * n2]; });
+                            [&](int gg, int n2) { return src[n1b + gg + N1 * n2]; });
   }
 
   const float inv_n = ldexpf(1.f, -P.logN) / (float)P.f;
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
       float ul[4], ur[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int64_t n = pos(h + j);
+        const int n = pos(h + j);
         ul[j] = ur[j] = 0.f;
         if (live(h + j) && n < P.L) {
           ul[j] = P.u[n];
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int64_t n = pos(h + j);
+        const int n = pos(h + j);
         if (!live(h + j) || n >= P.L) continue;
         const float2 yb = unscale(col[pidx(row_of(h + j))], inv_uh);
         if (MODE == COL_INV_OUT_KEEP) P.T2[n] = yb;
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
       float gl[4], gr[4], ul[4], ur[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int64_t n = pos(h + j);
+        const int n = pos(h + j);
         yb[j] = make_float2(0.f, 0.f);
         gl[j] = gr[j] = ul[j] = ur[j] = 0.f;
         if (live(h + j) && n < P.L) {
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
       float gl[4], gr[4], um[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int64_t n = pos(h + j);
+        const int n = pos(h + j);
         gl[j] = gr[j] = um[j] = 0.f;
         if (live(h + j) && n < P.L) {
           gl[j] = P.dy[n];
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int64_t n = pos(h + j);
+        const int n = pos(h + j);
         if (!live(h + j) || n >= P.L) continue;
         const float2 dw = unscale(col[pidx(row_of(h + j))], inv_dh);
         P.du[n] = wd * gl[j] + dw.x + um[j];
@@ -206,9 +206,9 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
 #pragma unroll 4
     for (int s = 0; s < kSlots; ++s) {
       if (!live(s)) continue;
-      const int64_t n = pos(s);
-      int64_t j = -1;
-      if (n < (int64_t)P.n0 + P.Nh) j = n - P.n0;
+      const int n = pos(s);
+      int j = -1;
+      if (n < P.n0 + P.Nh) j = n - P.n0;
       else if (n >= N + P.n0) j = n - N - P.n0;
       if (j >= 0 && j < P.Nh) {
         // dL/dh[t] = sum_n dL/dy_bar[n] u[n - t] is identically zero for lags t >= L: store the exact zero
@@ -293,14 +293,14 @@ __global__ void __launch_bounds__(kScaleThreads) k_chan_scale(LaunchCtx c, const
         acc[1] += b * b;
       }
   } else {
-    const int64_t N = fft_len(P);
+    const int N = fft_len(P);
     const int n = (P.Nh + 31) >> 5;             // every 32nd tap
     for (int i0 = 0; i0 < n; i0 += kScaleTile) {
       __syncthreads();
 #pragma unroll
       for (int j = 0; j < kScaleBatch; ++j) {
         const int i = i0 + t + j * kScaleThreads;
-        const int64_t at = (int64_t)32 * i + P.n0;
+        const int at = 32 * i + P.n0;
         if (i < n) tile[t + j * kScaleThreads] = tap_at(P, at >= 0 ? at : N + at, N);
       }
       __syncthreads();

@@ -36,7 +36,8 @@ __host__ __device__ constexpr int col_stride(int N2, int G) { return ((N2 + (N2 
 __device__ __forceinline__ int mirror_pos(int k2, int k1, int N1) { return k2 == 0 ? (k1 ? N1 - k1 : 0) : (N1 - 1 - k1); }
 
 __device__ __forceinline__ int rows_len(const ProcDev& P) { return P.f << P.logN1; }
-__device__ __forceinline__ int64_t fft_len(const ProcDev& P) { return (int64_t)P.f << P.logN; }
+// transform sizes fit 2^26, so every position of a grid is an int
+__device__ __forceinline__ int fft_len(const ProcDev& P) { return P.f << P.logN; }
 
 // Transposition twiddle exp(-+2 pi i m / N), m < N: the power-of-two tables, times exp(-2 pi i (m mod f) / N)
 // when N = f 2^logN, f = 3 or 5.
@@ -60,9 +61,9 @@ __device__ __forceinline__ void row_fft(float2* d, const ProcDev& P, int nb, int
 }
 
 // Tap value of the stereo FIR at circular position n (time n, or n - N for the negative taps).
-__device__ __forceinline__ float2 tap_at(const ProcDev& P, int64_t n, int64_t N) {
-  int64_t j;
-  if (n < (int64_t)P.n0 + P.Nh) j = n - P.n0;
+__device__ __forceinline__ float2 tap_at(const ProcDev& P, int n, int N) {
+  int j;
+  if (n < P.n0 + P.Nh) j = n - P.n0;
   else if (n >= N + P.n0) j = n - N - P.n0;
   else return make_float2(0.f, 0.f);
   if (j < 0 || j >= P.Nh) return make_float2(0.f, 0.f);
@@ -94,8 +95,8 @@ __device__ __forceinline__ void load_rows_fft(float2* s, const float2* src, int 
                                               const Tables& tab) {
   const int N1 = rows_len(P), rs = pstride(N1);
   const int nr = a == b ? 1 : 2;
-  const float2* ra = src + (int64_t)a * N1;
-  const float2* rb = src + (int64_t)b * N1;
+  const float2* ra = src + a * N1;
+  const float2* rb = src + b * N1;
   row_fft<false>(s, P, nr, rs, tab, [=](int slot, int k1) { return (slot ? rb : ra)[k1]; });
 }
 
@@ -121,8 +122,8 @@ __device__ __forceinline__ void inv_rows_store(float2* o, float2* dst, int a, in
                                                const Tables& tab, const float2* tt, LD ld = LD()) {
   const int N1 = rows_len(P), rs = pstride(N1), logT = min(6, __ffs(N1) - 1);
   const int nr = a == b ? 1 : 2;
-  float2* da = dst + (int64_t)a * N1;
-  float2* db = dst + (int64_t)b * N1;
+  float2* da = dst + a * N1;
+  float2* db = dst + b * N1;
   __syncthreads();
   row_fft<true>(o, P, nr, rs, tab, ld, [=](int slot, int n1, float2 v) {
     const float2* t = tt + slot * kRowTwS;
@@ -140,7 +141,7 @@ __device__ __forceinline__ void inv_rows_store(float2* o, float2* dst, int a, in
 template <int NB, typename Ld, typename Op>
 __device__ __forceinline__ void for_mirror_pairs(int a, int b, int N1, Ld&& load, Op&& op) {
   const int qs = a == b ? 0 : pstride(N1);
-  using V = decltype(load(int64_t(0), int64_t(0)));
+  using V = decltype(load(0, 0));
   for (int k0 = threadIdx.x; k0 < N1; k0 += NB * blockDim.x) {
     V v[NB];
     int kk[NB], mk[NB];
@@ -150,11 +151,11 @@ __device__ __forceinline__ void for_mirror_pairs(int a, int b, int N1, Ld&& load
       kk[j] = k0 + j * blockDim.x;
       mk[j] = mirror_pos(a, kk[j], N1);
       ok[j] = kk[j] < N1 && !(a == b && mk[j] < kk[j]);
-      if (ok[j]) v[j] = load((int64_t)a * N1 + kk[j], (int64_t)b * N1 + mk[j]);
+      if (ok[j]) v[j] = load(a * N1 + kk[j], b * N1 + mk[j]);
     }
 #pragma unroll
     for (int j = 0; j < NB; ++j)
-      if (ok[j]) op(pidx(kk[j]), qs + pidx(mk[j]), (int64_t)a * N1 + kk[j], (int64_t)b * N1 + mk[j], v[j]);
+      if (ok[j]) op(pidx(kk[j]), qs + pidx(mk[j]), a * N1 + kk[j], b * N1 + mk[j], v[j]);
   }
 }
 

@@ -13,8 +13,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_row_fwd_hz(LaunchCtx c, cons
   const int N1 = rows_len(P), N2 = 1 << P.logN2, rs = pstride(N1);
   const int a = it.idx, b = (N2 - it.idx) & (N2 - 1);
   const int nr = a == b ? 1 : 2;
-  float2* ha = P.Hz + (int64_t)a * N1;
-  float2* hb = P.Hz + (int64_t)b * N1;
+  float2* ha = P.Hz + a * N1;
+  float2* hb = P.Hz + b * N1;
   // global in, global out: the first pass reads the rows, the last writes them (the passes between hold
   // barriers, so every read precedes every write)
   row_fft<false>(sm, P, nr, rs, c.tab, [=](int slot, int k1) { return (slot ? hb : ha)[k1]; },
@@ -36,8 +36,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_row_conv(LaunchCtx c, const 
   row_tw_init(tt, P, a, b, c.tab);
   float2* s = sm;
   load_rows_fft(s, P.T1, a, b, P, c.tab);
-  for_mirror_pairs<4>(a, b, N1, [&](int64_t gP, int64_t gQ) { return HzPair{P.Hz[gP], P.Hz[gQ]}; },
-                      [&](int pP, int pQ, int64_t gP, int64_t gQ, const HzPair& v) {
+  for_mirror_pairs<4>(a, b, N1, [&](int gP, int gQ) { return HzPair{P.Hz[gP], P.Hz[gQ]}; },
+                      [&](int pP, int pQ, int gP, int gQ, const HzPair& v) {
     const float2 zP = s[pP], zQ = s[pQ];
     float2 AP, BP, AQ, BQ;
     fir_ab(v.hP, v.hQ, AP, BP);

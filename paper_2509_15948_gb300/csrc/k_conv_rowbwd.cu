@@ -34,8 +34,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_row_bwd2(LaunchCtx c, const 
   row_tw_init(tt, P, a, b, c.tab);
   load_rows_fft(s, P.T2, a, b, P, c.tab);
   for_mirror_pairs<4>(a, b, N1,
-                      [&](int64_t gP, int64_t gQ) { return HzUPair{P.Hz[gP], P.Hz[gQ], P.T1[gP], P.T1[gQ]}; },
-                      [&](int pP, int pQ, int64_t gP, int64_t gQ, const HzUPair& v) {
+                      [&](int gP, int gQ) { return HzUPair{P.Hz[gP], P.Hz[gQ], P.T1[gP], P.T1[gQ]}; },
+                      [&](int pP, int pQ, int gP, int gQ, const HzUPair& v) {
     const float2 dzP = s[pP], dzQ = s[pQ];
     float2 AP, BP, AQ, BQ;
     fir_ab(v.hP, v.hQ, AP, BP);
@@ -48,8 +48,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_row_bwd2(LaunchCtx c, const 
   inv_rows_store(s, P.T2, a, b, P, c.tab, tt);
   // the dH rows written to T1 become visible to the whole block at the barrier that opens the second inverse
   // transform, which reads them back from T1 in its first pass
-  const float2* ta = P.T1 + (int64_t)a * N1;
-  const float2* tb = P.T1 + (int64_t)b * N1;
+  const float2* ta = P.T1 + a * N1;
+  const float2* tb = P.T1 + b * N1;
   inv_rows_store(s, P.T1, a, b, P, c.tab, tt, [=](int slot, int k1) { return (slot ? tb : ta)[k1]; });
 }
 

@@ -301,6 +301,32 @@ __device__ __forceinline__ int divF(int x) {
 }
 __device__ __forceinline__ int div3(int x) { return divF<3>(x); }
 
+// Elements i, i + step, ... of one transform in the padded layout: with a step that is a multiple of 16 every address is
+// the first plus a multiple of the padded step (known at compile time in the unrolled sequences), otherwise each is
+// padded on its own.
+template <int R>
+__device__ __forceinline__ void load_padded(float2 (&v)[R], const float2* src, int i, int step) {
+  if ((step & 15) == 0) {
+    src += pidx(i);
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = src[r * (step + (step >> 4))];
+  } else {
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = src[pidx(i + r * step)];
+  }
+}
+template <int R>
+__device__ __forceinline__ void store_padded(const float2 (&v)[R], float2* dst, int i, int step) {
+  if ((step & 15) == 0) {
+    dst += pidx(i);
+#pragma unroll
+    for (int r = 0; r < R; ++r) dst[r * (step + (step >> 4))] = v[r];
+  } else {
+#pragma unroll
+    for (int r = 0; r < R; ++r) dst[pidx(i + r * step)] = v[r];
+  }
+}
+
 // First pass (p = 1, no twiddles): butterfly i < 2^a reads x[i + r 2^a], writes F i + q.
 template <bool INV, int F, class LD = SmemIO>
 __device__ __forceinline__ void passF(float2* __restrict__ d, int a, int nb, int bs, LD ld = LD()) {
@@ -318,9 +344,7 @@ __device__ __forceinline__ void passF(float2* __restrict__ d, int a, int nb, int
 #pragma unroll
         for (int r = 0; r < F; ++r) v[s][r] = ld(b, i + r * MR);
       } else {
-        const float2* src = d + b * bs;
-#pragma unroll
-        for (int r = 0; r < F; ++r) v[s][r] = src[pidx(i + r * MR)];
+        load_padded<F>(v[s], d + b * bs, i, MR);
       }
       dftF<INV, F>(v[s]);
       ob[s] = b * bs;
@@ -354,9 +378,7 @@ __device__ __forceinline__ void passm(float2* __restrict__ d, int a, int nb, int
     if (it < total) {
       const int b = divF<F>(it >> (a - LOGR)), i = it - b * MR;   // it / MR, MR = F 2^(a - LOGR)
       const int k = i - p * divF<F>(i >> lp2);                      // i mod p, p = F 2^lp2
-      const float2* src = d + b * bs;
-#pragma unroll
-      for (int r = 0; r < R; ++r) v[s][r] = src[pidx(i + r * MR)];
+      load_padded<R>(v[s], d + b * bs, i, MR);
       if (k) twiddle<INV, R>(v[s], ptwf + ptwf_base(F, a, lp2) + k, p);
       dftR<INV, R>(v[s]);
       ob[s] = b * bs + (i - k) * R + k;
@@ -372,9 +394,7 @@ __device__ __forceinline__ void passm(float2* __restrict__ d, int a, int nb, int
 #pragma unroll
         for (int q = 0; q < R; ++q) st(b, e0 + q * p, v[s][q]);
       } else {
-        float2* dst = d + b * bs;
-#pragma unroll
-        for (int q = 0; q < R; ++q) dst[pidx(e0 + q * p)] = v[s][q];
+        store_padded<R>(v[s], d + b * bs, e0, p);
       }
     }
   }
