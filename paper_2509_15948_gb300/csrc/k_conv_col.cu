@@ -37,6 +37,50 @@ __device__ __forceinline__ void col_tw_init(float2* ctw, const ProcDev& P, int n
   }
 }
 
+// Sums of a tile in the order of 512 threads whatever the block size, so that a node's energies and dL/dw do not depend on
+// it: thread t of a smaller block stands for threads t + i blockDim, whose rows are its slots s = i (mod 512 / blockDim)
+// and whose sums it keeps apart (four at most; tiles of 1,024 elements or fewer add the rest in slot order).
+struct TileSums {
+  int gm;                                    // min(512 / blockDim, 4) - 1
+  __device__ __forceinline__ TileSums() : gm(min(kColThreads / (int)blockDim.x, 4) - 1) {}
+  template <int NV>
+  __device__ __forceinline__ void add(float (&acc)[4][NV], int j, int v, float x) const {   // j: slot mod 4
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if ((j & gm) == k) acc[k][v] += x;
+  }
+  // fma of the same
+  template <int NV>
+  __device__ __forceinline__ void add_mul(float (&acc)[4][NV], int j, int v, float x, float y) const {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if ((j & gm) == k) acc[k][v] += x * y;
+  }
+  template <int NV>
+  __device__ __forceinline__ void total(float (&acc)[4][NV], float* red /* NV * 32 */, float* out) const {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5, n = nw * (gm + 1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        if (k > gm) continue;
+        float x = acc[k][v];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+        if (lane == 0) red[v * 32 + k * nw + wid] = x;
+      }
+    __syncthreads();
+    if (wid == 0)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        float x = lane < n ? red[v * 32 + lane] : 0.f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+        if (lane == 0) out[v] = x;
+      }
+  }
+};
+
 template <int MODE>
 __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item* __restrict__ items) {
   extern __shared__ float2 sm[];
@@ -101,7 +145,8 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
   auto unscale = [](float2 v, float2 s) { return make_float2(v.x * s.x, v.y * s.y); };
   if (kOut) {
     const float w = dry_wet_w(c, P.qidx), wd = dry_wet_d(c, P.qidx);
-    float acc[2] = {0.f, 0.f};
+    const TileSums ts;
+    float acc[4][2] = {};
 #pragma unroll 1
     for (int h = 0; h < kSlots; h += 4) {
       float ul[4], ur[4];
@@ -123,12 +168,12 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
         P.y[n] = w * yb.x + wd * ul[j];
         P.y[P.ld + n] = w * yb.y + wd * ur[j];
         const float ym = yb.x + yb.y, um = ul[j] + ur[j];
-        acc[0] += ym * ym;
-        acc[1] += um * um;
+        ts.add_mul(acc, j, 0, ym, ym);
+        ts.add_mul(acc, j, 1, um, um);
       }
     }
     float out[2];
-    block_sum<2>(acc, red, out);
+    ts.total(acc, red, out);
     if (threadIdx.x == 0) {
       P.fpart[it.idx * kNPart + 0] = out[0];
       P.fpart[it.idx * kNPart + 1] = out[1];
@@ -140,7 +185,8 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
     // Retained spectra: y_bar is read in natural order from T2; otherwise it is the inverse column FFT above.
     const float w = dry_wet_w(c, P.qidx);
     const float c1 = P.stats[2];
-    float acc[1] = {0.f};
+    const TileSums ts;
+    float acc[4][1] = {};
 #pragma unroll 1
     for (int h = 0; h < kSlots; h += 4) {
       float2 yb[4];
@@ -161,14 +207,14 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         if (!live(h + j)) continue;
-        acc[0] += gl[j] * (yb[j].x - ul[j]) + gr[j] * (yb[j].y - ur[j]);
+        ts.add(acc, j, 0, gl[j] * (yb[j].x - ul[j]) + gr[j] * (yb[j].y - ur[j]));
         const float gm = c1 * (yb[j].x + yb[j].y);
         // rows past the signal are zero (gl = gr = 0 and y_bar = 0 there)
         col[pidx(row_of(h + j))] = make_float2(sd.x * (w * gl[j] + gm), sd.y * (w * gr[j] + gm));
       }
     }
     float out[1];
-    block_sum<1>(acc, red, out);   // also acts as the barrier before the FFT
+    ts.total(acc, red, out);   // also acts as the barrier before the FFT
     if (threadIdx.x == 0) P.bpart[it.idx * kNPart + 0] = out[0];
     fft_p_io<false, 1, true>(sm, logN2, G, cs, c.tab.ptw, fftp::SmemIO(), tw_store(P.T2));
     return;

@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_loss_frames(LaunchCtx c, co
     // pairs (frame, band) go band by band, so that the threads of a warp run over equally long bands and read the same
     // weights, and a weight and its bin serve all four channels.  (One thread per value, resp. one warp per pair with 20
     // entries on average for its 32 lanes, was 60 % of the kernel's instructions.)
+    const bool wide = R.band_beg[nbands] >= 16 * nbands;
     float* yv = reinterpret_cast<float*>(sm + kFrameBuf);
     const int pairs = nb * nbands;
     const float inv_nb = 1.f / (float)nb;   // e / nb = floor((e + 1/2) inv_nb): pairs < 2^16
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_loss_frames(LaunchCtx c, co
       const int r = b + (f & rot);
       return f * nbands + (r >= nbands ? r - nbands : r);
     };
-    if (R.band_beg[nbands] >= 16 * nbands) {
+    if (wide) {
       // wide bands: eight lanes per pair.  Lane l holds the sums of entries l + 8 i (mod 32), i < 4, which are then added
       // as a warp would over its lanes with xor 16, 8, 4, 2, 1.
       const int l8 = threadIdx.x & 7;
@@ -202,37 +203,60 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_loss_frames(LaunchCtx c, co
       }
     }
     __syncthreads();
-    // the values in frame order, target and kept values coalesced; a thread only ever adds terms of one channel
+    // the values in frame order, target and kept values coalesced.  The sums go in fixed chains of one channel each: narrow
+    // bands, thread t adds values t, t + 512, ...; wide ones, lane c < 4 of a warp adds channel c of every 16th pair,
+    // after all threads have put the terms where the frames were.
+    const int row = nbands * 4, total = nb * row;
+    float *t0v = reinterpret_cast<float*>(sm), *t1v = t0v + total;   // wide: total <= 2,048
     float acc0 = 0.f, acc1 = 0.f;
     const int mych = threadIdx.x & 3;
     {
-      const int row = nbands * 4, total = nb * row;
       const float inv_row = 1.f / (float)row;
       const size_t base = (size_t)t0 * row;
       constexpr int kAhead = 4;
       for (int e0 = threadIdx.x; e0 < total; e0 += kAhead * blockDim.x) {
         float yt[kAhead];
-        int at[kAhead];
-#pragma unroll
-        for (int j = 0; j < kAhead; ++j) {
-          const int e = e0 + j * blockDim.x, f = (int)((e + 0.5f) * inv_row);
-          const int r = e - f * row - 4 * (f & rot);
-          at[j] = f * row + (r < 0 ? r + row : r);
-          yt[j] = mode != 0 && e < total ? Yt[base + at[j]] : 0.f;
-        }
 #pragma unroll
         for (int j = 0; j < kAhead; ++j) {
           const int e = e0 + j * blockDim.x;
+          yt[j] = mode != 0 && e < total ? Yt[base + e] : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+          const int e = e0 + j * blockDim.x, f = (int)((e + 0.5f) * inv_row);
           if (e >= total) continue;
-          const float yh = yv[e];
-          if (mode == 3) Yk[base + at[j]] = yh;
+          const int r = e - f * row + 4 * (f & rot);
+          const float yh = yv[f * row + (r >= row ? r - row : r)];
+          if (mode == 3) Yk[base + e] = yh;
           if (mode == 0) {
-            Yt[base + at[j]] = yh;
-            acc0 += yh * yh;
+            Yt[base + e] = yh;
+            if (wide) t0v[e] = yh;
+            else acc0 += yh * yh;
           } else {
-            acc0 += fabsf(logf(yt[j] + kLogEps) - logf(yh + kLogEps));
-            const float d = yt[j] - yh;
-            acc1 += d * d;
+            const float dl = fabsf(logf(yt[j] + kLogEps) - logf(yh + kLogEps)), d = yt[j] - yh;
+            if (wide) {
+              t0v[e] = dl;
+              t1v[e] = d;
+            } else {
+              acc0 += dl;
+              acc1 += d * d;
+            }
+          }
+        }
+      }
+    }
+    if (wide) {
+      __syncthreads();
+      if ((threadIdx.x & 31) < 4) {
+#pragma unroll 4
+        for (int e = threadIdx.x >> 5; e < pairs; e += blockDim.x >> 5) {
+          const float x0 = t0v[4 * e + mych];
+          if (mode == 0) {
+            acc0 += x0 * x0;
+          } else {
+            const float x1 = t1v[4 * e + mych];
+            acc0 += x0;
+            acc1 += x1 * x1;
           }
         }
       }
