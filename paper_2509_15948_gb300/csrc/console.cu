@@ -913,6 +913,11 @@ void loss_forward(mg_console* c, const LaunchCtx& x, int mode, float* out_losses
 }
 
 void backward_pass(mg_console* c, const LaunchCtx& x) {
+  if (!c->fir[fir_slot(T_D)].procs.h.empty()) {   // the delay adjoints' powers of z, beside the loss adjoint
+    StageScope scope(c, T_D);
+    const LaunchCtx y = fork(c, x, T_D, c->adj_pending);
+    run_procs(c, F_FIR_ADJ, c->fir[fir_slot(T_D)].procs, [&](const int* p, int n) { launch_dly_pow(y, p, n); });
+  }
   {
     StageScope scope(c, 7);
     auto& L = c->loss_items;
@@ -1535,7 +1540,7 @@ size_t layout_arena(mg_console* c, const mg_console_desc* d, size_t* shared_scra
       p.o_ybar = b.take((size_t)2 * p.ld * sizeof(float));
       p.o_eqg = b.take((size_t)p.nfrows * kEqOsM * sizeof(float2));
     }
-    if (p.type == T_D) p.o_aux = b.take((2 * kDlyTaps * kDlyFir + 2 * kDlyTaps) * sizeof(float));
+    if (p.type == T_D) p.o_aux = b.take(kDlyAuxFloats * sizeof(float));
     if (p.type == T_C || p.type == T_N) p.o_aux = b.take((size_t)p.ld * sizeof(float));   // dL/dg per sample
     if (p.type == T_R) {
       const int ng = (p.nframes + kRevFG - 1) / kRevFG;

@@ -92,8 +92,11 @@ __global__ void __launch_bounds__(kEqFirThreads) k_eq_fir_adj(LaunchCtx c, const
 // ------------------------------------------------------------------------------------------------
 // multitap delay
 // ------------------------------------------------------------------------------------------------
-// aux layout: [2][20][39] c_m taps, then [2][20] integer delays (stored as int).
+// aux layout: [2][20][39] c_m taps, then [2][20] integer delays (stored as int), then [2][20][3] complex z_m^D,
+// z_m^(D-1), z_m of the z clamped to the unit disk (k_dly_pow).
 constexpr int kDlyAuxC = 2 * kDlyTaps * kDlyFir;
+constexpr int kDlyAuxZ = kDlyAuxC + 2 * kDlyTaps;
+static_assert(kDlyAuxZ % 2 == 0 && kDlyAuxFloats == kDlyAuxZ + 2 * kDlyTaps * 6, "float2 entries, as the arena reserves");
 
 __device__ __forceinline__ int dly_slot(double fs) { return (int)llrint(0.1 * fs); }
 
@@ -193,13 +196,38 @@ __device__ __noinline__ float2 pole_sum(float2 a, int D) {
   return make_float2((float)((nr * qr + ni * qi) * k), (float)((ni * qr - nr * qi) * k));
 }
 
+// Powers of the clamped z for the adjoint (Eq. 18's derivative), in double: CTA (node, channel and exponent), the angle
+// on one warp, the radius on the other, a tap per lane.  An SM does two double-precision operations per cycle and a warp
+// instruction costs the same with one lane as with 32: with five lanes of every adjoint block doing the powers of
+// their own tap, they were two thirds of that kernel (12 delays x 7 s: block 917 -> 888 us).
+__global__ void __launch_bounds__(64) k_dly_pow(LaunchCtx c, const int* __restrict__ procs) {
+  __shared__ double ang[2][kDlyTaps], rad[kDlyTaps];
+  const ProcDev& P = c.procs[procs[blockIdx.x]];
+  const int ch = blockIdx.y >> 1, part = blockIdx.y & 1, m = threadIdx.x & 31;
+  const int D = dly_slot(c.fs);
+  const float* z = P.p + (ch * kDlyTaps + m) * kDlyPer;
+  float2* out = reinterpret_cast<float2*>(P.aux + kDlyAuxZ) + (ch * kDlyTaps + m) * 3;
+  if (m < kDlyTaps) {
+    const double zr = z[0], zi = z[1];
+    const double rz = sqrt(zr * zr + zi * zi);
+    const double sc = rz > 1.0 ? 1.0 / rz : 1.0;
+    const double hr = zr * sc, hi = zi * sc, hrad = rz * sc;
+    if (threadIdx.x < 32) {
+      sincos((double)(D - part) * atan2(hi, hr), &ang[1][m], &ang[0][m]);
+    } else {
+      rad[m] = hrad > 0.0 ? pow(hrad, (double)(D - part)) : 0.0;
+      if (part == 0) out[2] = make_float2((float)hr, (float)hi);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < kDlyTaps) out[part] = make_float2((float)(rad[m] * ang[0][m]), (float)(rad[m] * ang[1][m]));
+}
+
 __global__ void __launch_bounds__(256) k_dly_adj(LaunchCtx c, const Item* __restrict__ items) {
   __shared__ float cm[kDlyFir];
   __shared__ float dc[kDlyFir];
   __shared__ float red[2 * 32];
   __shared__ float gsum[2];
-  __shared__ float2 zsh[3];   // z^D, z^(D-1), z clamped to the unit disk
-  __shared__ double zpow[6];  // cos, sin of D arg z and of (D - 1) arg z; |z|^D, |z|^(D-1)
   const Item it = items[blockIdx.x];
   const ProcDev& P = c.procs[it.proc];
   const int ch = it.idx / kDlyTaps, m = it.idx % kDlyTaps;
@@ -213,27 +241,6 @@ __global__ void __launch_bounds__(256) k_dly_adj(LaunchCtx c, const Item* __rest
     cm[threadIdx.x] = P.aux[(ch * kDlyTaps + m) * kDlyFir + threadIdx.x];
     dc[threadIdx.x] = dh[d + threadIdx.x];   // tap time d + j - 19 -> index d + j (first tap at -19)
   }
-  // (b, scalars) the powers of z in double, once per block, each factor on a warp of its own (FP64 is slow, and
-  // lanes of one warp would take their branches one after the other)
-  if ((threadIdx.x & 31) == 0 && threadIdx.x < 5 * 32) {
-    const int part = threadIdx.x >> 5;
-    const double zr = pz[0], zi = pz[1];
-    const double rz = sqrt(zr * zr + zi * zi);
-    const double sc = rz > 1.0 ? 1.0 / rz : 1.0;
-    const double hr = zr * sc, hi = zi * sc, hrad = rz * sc;
-    if (part < 2) {
-      sincos((double)(D - part) * atan2(hi, hr), &zpow[2 * part + 1], &zpow[2 * part]);
-    } else if (part < 4) {
-      zpow[2 + part] = hrad > 0.0 ? pow(hrad, (double)(D - (part - 2))) : 0.0;
-    } else {
-      zsh[2] = make_float2((float)hr, (float)hi);
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < 2) {
-    const double r = zpow[4 + threadIdx.x];
-    zsh[threadIdx.x] = make_float2((float)(r * zpow[2 * threadIdx.x]), (float)(r * zpow[2 * threadIdx.x + 1]));
-  }
   __syncthreads();
   // (a) log-magnitudes of c_m
   if (threadIdx.x <= kDlyHalf) {
@@ -246,8 +253,9 @@ __global__ void __launch_bounds__(256) k_dly_adj(LaunchCtx c, const Item* __rest
     gz[2 + k] = expf(pz[2 + k]) * (k == 0 ? 1.f : 2.f) * (1.f / kDlyFir) * acc;
   }
   // (b) angular frequency
-  const float2 zD1 = zsh[1], zh = zsh[2];
-  const float2 omz = make_float2(1.f - zsh[0].x, -zsh[0].y);
+  const float2* zp = reinterpret_cast<const float2*>(P.aux + kDlyAuxZ) + (ch * kDlyTaps + m) * 3;
+  const float2 zD = zp[0], zD1 = zp[1], zh = zp[2];
+  const float2 omz = make_float2(1.f - zD.x, -zD.y);
   double accd[2] = {0.0, 0.0};
   for (int q = threadIdx.x; q < D; q += blockDim.x) {
     float G = 0.f;
@@ -535,6 +543,9 @@ void launch_eq_fir_adj(const LaunchCtx& c, const int* procs, int n) {
 }
 void launch_dly_prep(const LaunchCtx& c, const int* procs, int n) {
   if (n) k_dly_prep<<<n, 256, 0, c.stream>>>(c, procs);
+}
+void launch_dly_pow(const LaunchCtx& c, const int* procs, int n) {
+  if (n) k_dly_pow<<<dim3(n, 4), 64, 0, c.stream>>>(c, procs);
 }
 void launch_dly_fir(const LaunchCtx& c, const Item* items, int n) {
   if (n) k_dly_fir<<<n, 256, 0, c.stream>>>(c, items);

@@ -23,6 +23,7 @@ constexpr int kDlyFir = 39;                // Sec. 3.7
 constexpr int kDlyHalf = 19;
 constexpr int kDlyTaps = 20;
 constexpr int kDlyPer = 22;                // Re z, Im z, 20 log-magnitudes
+constexpr int kDlyAuxFloats = 2 * kDlyTaps * (kDlyFir + 1 + 6);   // per delay: c_m, positions, powers of z (k_fir.cu)
 constexpr int kRevFft = 384;               // Sec. 3.4
 constexpr int kRevHop = 192;
 constexpr int kRevBins = 193;
@@ -175,6 +176,7 @@ void launch_dyn_bwd(const LaunchCtx&, const Item* items, int n);
 void launch_eq_fir(const LaunchCtx&, const int* procs, int n);
 void launch_eq_fir_adj(const LaunchCtx&, const int* procs, int n);
 void launch_dly_prep(const LaunchCtx&, const int* procs, int n);
+void launch_dly_pow(const LaunchCtx&, const int* procs, int n);
 void launch_dly_fir(const LaunchCtx&, const Item* items, int n);
 void launch_dly_adj(const LaunchCtx&, const Item* items, int n);
 void launch_rev_fir(const LaunchCtx&, const Item* items, int n);
