@@ -139,10 +139,13 @@ __global__ void __launch_bounds__(256) k_dly_fir(LaunchCtx c, const Item* __rest
   __syncthreads();
   const int j = it.idx * blockDim.x + threadIdx.x;
   if (j >= P.Nh) return;
-  const int n = j + P.n0;
+  // tap m lies in the slot [m D, (m + 1) D) (or, for a z that is not a number, the one before), so its window reaches n
+  // for at most three m (all twenty were tried before: 25 us on 20 nodes)
+  const int n = j + P.n0, D = dly_slot(c.fs);
+  const int m0 = n > kDlyHalf ? (n - kDlyHalf) / D : 0, m1 = min(kDlyTaps - 1, (n + kDlyHalf) / D + 1);
   for (int ch = 0; ch < 2; ++ch) {
     float acc = 0.f;
-    for (int m = 0; m < kDlyTaps; ++m) {
+    for (int m = m0; m <= m1; ++m) {
       const int o = n - dpos[ch * kDlyTaps + m];
       if (o >= -kDlyHalf && o <= kDlyHalf) acc += P.aux[(ch * kDlyTaps + m) * kDlyFir + o + kDlyHalf];
     }
@@ -413,15 +416,21 @@ __global__ void __launch_bounds__(512) k_rev_fir(LaunchCtx c, const Item* __rest
   const int F = P.nframes, ng = (F + kRevFG - 1) / kRevFG;
   const int grp = it.idx, t0 = grp * kRevFG, tb = t0 - 1;
   constexpr int NF = kRevFG + 1;
+  // H0 and H_delta of every bin once (the softplus was half of the kernel when every frame formed it again)
+  __shared__ float2 hd[2][kRevParams];
+  for (int e = threadIdx.x; e < 2 * kRevParams; e += blockDim.x) {
+    const int x = e / kRevParams, k = e - x * kRevParams;
+    const float* px = P.p + x * 2 * kRevParams;      // [x][H0, p_delta][192]
+    hd[x][k] = make_float2(px[k], -0.05f * softplusf_(px[kRevParams + k]));
+  }
+  __syncthreads();
   for (int e = threadIdx.x; e < NF * kRevBins; e += blockDim.x) {
     const int f = e / kRevBins, k = e % kRevBins, t = tb + f;
     float2 hm = make_float2(0.f, 0.f), hs = hm;
     if (t >= 0 && t < F) {
       const int kk = k < kRevParams ? k : kRevParams - 1;
-      const float* pm = P.p;                          // [x][H0, p_delta][192]
-      const float* ps = P.p + 2 * kRevParams;
-      const float mm = expf(pm[kk] + (float)t * (-0.05f * softplusf_(pm[kRevParams + kk])));
-      const float ms = expf(ps[kk] + (float)t * (-0.05f * softplusf_(ps[kRevParams + kk])));
+      const float mm = expf(hd[0][kk].x + (float)t * hd[0][kk].y);
+      const float ms = expf(hd[1][kk].x + (float)t * hd[1][kk].y);
       hm = cscale(P.nspec[((size_t)0 * F + t) * kRevBins + k], mm);
       hs = cscale(P.nspec[((size_t)1 * F + t) * kRevBins + k], ms);
     }
@@ -455,7 +464,7 @@ __global__ void __launch_bounds__(512) k_rev_fir(LaunchCtx c, const Item* __rest
 // item = (node, grp): frames t in [t0, t0 + 16); partial sums of dL/dH0 and dL/dp_delta per bin, for mid and
 // side.  dframe_x[j] = w[j] dh_x[192 t + j] / env (dh_m = dh_l + dh_r, dh_s = dh_l - dh_r), packed forward DFT,
 // dRe H[k] = c_k Re F[k] / 384, dIm H[k] = c_k Im F[k] / 384 (c_k = 1 at DC / Nyquist where Im is unused).
-__global__ void __launch_bounds__(512) k_rev_adj(LaunchCtx c, const Item* __restrict__ items) {
+__global__ void __launch_bounds__(512, 2) k_rev_adj(LaunchCtx c, const Item* __restrict__ items) {
   extern __shared__ float2 sm[];
   const Item it = items[blockIdx.x];
   const ProcDev& P = c.procs[it.proc];
@@ -486,6 +495,7 @@ __global__ void __launch_bounds__(512) k_rev_adj(LaunchCtx c, const Item* __rest
     const float dhd = -0.05f / (1.f + expf(-pd[kk]));    // d H_delta / d p_delta
     const float ck = (k == 0 || k == kRevBins - 1) ? 1.f : 2.f;
     float a0 = 0.f, a1 = 0.f;
+#pragma unroll 4   // the frames' noise spectra in flight together
     for (int f = 0; f < nf; ++f) {
       const float2 A = sm[f * kRevFft + k], B = sm[f * kRevFft + ((kRevFft - k) % kRevFft)];
       float2 Fx;
