@@ -49,12 +49,12 @@ struct TileSums {
     for (int k = 0; k < 4; ++k)
       if ((j & gm) == k) acc[k][v] += x;
   }
-  // fma of the same
+  // the same of a product, fused (left to the compiler the shared product is rounded on its own)
   template <int NV>
   __device__ __forceinline__ void add_mul(float (&acc)[4][NV], int j, int v, float x, float y) const {
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      if ((j & gm) == k) acc[k][v] += x * y;
+      if ((j & gm) == k) acc[k][v] = __fmaf_rn(x, y, acc[k][v]);
   }
   template <int NV>
   __device__ __forceinline__ void total(float (&acc)[4][NV], float* red /* NV * 32 */, float* out) const {
