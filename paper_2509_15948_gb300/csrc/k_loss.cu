@@ -9,12 +9,11 @@
 // transposed Mel CSR, to the complex bins through |X|, to the packed Hermitian spectrum, and through one
 // inverse FFT to the windowed frame; a gather kernel overlap-adds the frames of all resolutions.
 //
-// What bounds it: with two CTAs per SM (64 registers, 69-94 KB) a work item is latency.  The Mel sums and the adjoint's
-// band values went one (frame, band) after the other, each waiting for its own table and target loads and for 20
-// shuffles, 45 us per wave of CTAs whatever the resolution.  Four values of a thread or warp now go together with
-// the target loaded before the sums, the warp sums take 7 shuffles, the four channels of a bin share its weights,
-// and all resolutions are one launch.  On one 30 s mix forward, adjoint and overlap-add took 780 us, now 270.
-// Every sum keeps its order, so the losses and gradients keep their bits.
+// What bounds it: issue and latency of 32 warps per SM (two CTAs of 64 registers a thread and 95 KB; issue slots half
+// used).  Before, the Mel sums and the adjoint's band values went one (frame, band) after the other, each waiting for its
+// own table and target loads and for 20 shuffles, 45 us per wave of CTAs whatever the resolution and a launch for each.
+// All resolutions are one launch now, the sums go band by band with a weight for four channels, and the loss terms are one
+// coalesced pass: forward, adjoint and overlap-add of a 30 s mix took 780 us, now 414 (203, 183 and 28).  Every sum keeps its order, so the losses and gradients keep their bits.
 #include "mg_fftp.cuh"
 
 namespace mg {
