@@ -288,14 +288,6 @@ mg_status fail(mg_console* c, mg_status s, const std::string& msg) {
 // ------------------------------------------------------------------------------------------------
 // planning (host only)
 // ------------------------------------------------------------------------------------------------
-// Four-step split of N = f 2^logN into rows N1 = f 2^logN1 and columns N2 = 2^logN2; a split is valid when the
-// rows fit the row kernels (N1 <= 2048, 3072 with the factor 3, 2560 with the factor 5), a column tile holds at
-// least one column (N2 <= 8192) and both factors are at least 8 (16 for the rows, one radix-16 pass).
-bool split_ok(int f, int logN, int logN1) {
-  const int logN2 = logN - logN1;
-  const int max_a = f == 1 ? 11 : (f == 3 ? kPtw3MaxA : kPtw5MaxA);
-  return logN1 >= 4 && logN2 >= 3 && logN2 <= 13 && logN1 <= max_a;
-}
 void apply_split(HostProc& p, int logN1) {
   p.logN1 = logN1;
   p.logN2 = p.logN - logN1;

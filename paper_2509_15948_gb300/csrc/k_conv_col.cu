@@ -27,7 +27,6 @@ constexpr int kSlots = 16;
 // N2 / 64 <= 32 hi entries), both factors from the accurate table; column gg at ctw + gg * kColTwS.  The column
 // stride is 4 (mod 16) float2 so that the eight columns x four rows of a warp's lookups spread evenly over the
 // bank pairs.  Visible after the caller's next barrier.
-constexpr int kColTwS = 100;
 __device__ __forceinline__ void col_tw_init(float2* ctw, const ProcDev& P, int n1b, int G, int N2, const Tables& tab) {
   for (int e = threadIdx.x; e < G * kColTwS; e += blockDim.x) {
     const int gg = e / kColTwS, j = e - gg * kColTwS;

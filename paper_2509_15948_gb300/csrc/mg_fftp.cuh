@@ -44,6 +44,19 @@ constexpr int kPtw3MaxA = 10;
 constexpr int kPtw3Count = 12 * ((2 << kPtw3MaxA) - 2);
 constexpr int kPtw5MaxA = 9;
 constexpr int kPtw5Count = 20 * ((2 << kPtw5MaxA) - 2);
+
+// Four-step split of N = f 2^logN into rows N1 = f 2^logN1 and columns N2 = 2^logN2.  A split is admitted when the rows
+// fit the row kernels and their twiddle tables (N1 <= 2048, 3072 with the factor 3, 2560 with the factor 5), the columns
+// the transposition twiddles of the column passes (N2 <= 2^kMaxColLog), and both factors are at least 8 (16 for the rows, one
+// radix-16 pass).  A column's twiddles W(n1 k2) are 64 entries for k2 mod 64 and N2 / 64 for k2 / 64; kColTwS apart.
+constexpr int kMaxColLog = 11;
+constexpr int kColTwS = 100;
+static_assert(64 + ((1 << kMaxColLog) >> 6) <= kColTwS, "the longest admitted column has all its twiddles in its own table");
+inline bool split_ok(int f, int logN, int logN1) {
+  const int logN2 = logN - logN1;
+  const int max_a = f == 1 ? 11 : (f == 3 ? kPtw3MaxA : kPtw5MaxA);
+  return logN1 >= 4 && logN2 >= 3 && logN2 <= kMaxColLog && logN1 <= max_a;
+}
 __host__ __device__ constexpr int ptwf_base(int f, int a, int lp2) {
   return 4 * f * ((1 << a) - 2) + 4 * f * (((1 << lp2) - 1) / 15);
 }
