@@ -38,10 +38,11 @@ __device__ __forceinline__ void col_tw_init(float2* ctw, const ProcDev& P, int n
 
 // Sums of a tile in the order of 512 threads whatever the block size, so that a node's energies and dL/dw do not depend on
 // it: thread t of a smaller block stands for threads t + i blockDim, whose rows are its slots s = i (mod 512 / blockDim)
-// and whose sums it keeps apart (four at most; tiles of 1,024 elements or fewer add the rest in slot order).
+// and whose sums it keeps apart, four at most: a block has at least kColMinThreads threads, whatever its tile.
+constexpr int kColMinThreads = kColThreads / 4;
 struct TileSums {
-  int gm;                                    // min(512 / blockDim, 4) - 1
-  __device__ __forceinline__ TileSums() : gm(min(kColThreads / (int)blockDim.x, 4) - 1) {}
+  int gm;                                    // 512 / blockDim - 1
+  __device__ __forceinline__ TileSums() : gm(kColThreads / (int)blockDim.x - 1) {}
   template <int NV>
   __device__ __forceinline__ void add(float (&acc)[4][NV], int j, int v, float x) const {   // j: slot mod 4
 #pragma unroll
@@ -371,7 +372,7 @@ void launch_col(const LaunchCtx& c, const Item* items, int n, int maxN2G) {
   // one thread per 16 elements of the largest tile: with 512 threads and 70 KB whatever the tile, half (N2 = 512) to
   // three quarters (N2 = 256) of the threads sat at the barriers and two CTAs filled an SM (16 x 10 s step 3,555 ->
   // 3,293 us, 3.8 s crop of 24 tracks 2,137 -> 1,849 us)
-  const int threads = std::max(32, std::min(kColThreads, maxN2G / 16));
+  const int threads = std::max(kColMinThreads, std::min(kColThreads, maxN2G / 16));   // a power of two (see TileSums)
   const size_t smem = (size_t)(maxN2G + maxN2G / 16 + kColPad) * sizeof(float2);
   k_col<MODE><<<n, threads, smem, c.stream>>>(c, items);
 }
