@@ -124,6 +124,7 @@ struct Stage {
   ItemList elem_rev;             // c, n: chunk items in reverse order per node (the chained backward)
   ItemList chain_f, chain_b;     // c, n: the same chunks in rounds across nodes (batched launches)
   ItemList osf;                  // e: overlap-save blocks
+  bool beside = false;           // e: in a captured step the tap adjoints run beside the chain (see adjoint_rule)
   std::vector<LtiGroup> groups;  // e, r, d
 };
 
@@ -833,8 +834,7 @@ void stage_backward(mg_console* c, const LaunchCtx& x, Stage& s) {
       break;
     case T_E: {
       run_items(c, F_EQ_OS_BWD, s.osf, [&](const Item* it, int n) { launch_eq_os_bwd(x, it, n); });
-      // issued eagerly, the fork costs more than it hides (equalizer block 976 us with it, 922 without)
-      const LaunchCtx y = c->capturing ? fork(c, x, T_E, c->adj_pending) : x;
+      const LaunchCtx y = s.beside && c->capturing ? fork(c, x, T_E, c->adj_pending) : x;   // see adjoint_rule
       run_procs(c, F_FIR_ADJ, s.procs, [&](const int* p, int n) { launch_eq_dh_reduce(y, p, n); });
       run_procs(c, F_FIR_ADJ, s.procs, [&](const int* p, int n) { launch_eq_fir_adj(y, p, n); });
       break;
@@ -1237,6 +1237,26 @@ mg_status join_fir_lists(mg_console* c) {
   return MG_OK;
 }
 
+// Which equalizer stages fork their tap adjoints (about 35 us of launches of a few CTAs) in a captured step.  They hide
+// beside the stages that follow, but they cost more than they hide where the next equalizers' launch follows at once and
+// needs more than one of the two places that an SM has for k_eq_os_bwd (adjoints on some of them leave it another wave).
+// So they fork at the last equalizers, where other stages than gain/pan and imager lie between, or before at most one
+// block per SM.
+// Captured steps with the fork and without (tracks + subgroups, us): equalizers and gain/pan 4+1 x 2 s 217 and 241,
+// 12+4 x 3 s 355 and 308 (302 by this rule), 24+4 x 10 s 864 and 806 (797), 8+2 x 60 s 2,038 and 1,996 (1,982); with
+// compressors 12+4 x 3 s 318 and 346; all types 4+1 x 2 s 809 and 842, 12+4 x 3 s 1,345 and 1,330, 16+4 x 10 s 3,101
+// and 3,133.  Issued eagerly the fork is not sure to pay: compressors, gates and all below 24+4 x 3 s 614 and 655, but
+// equalizers and gain/pan 24+4 x 10 s 905 and 858, equalizers and reverbs 12+4 x 3 s 860 and 772; there is none.
+void adjoint_rule(mg_console* c) {
+  for (int k = 0; k < (int)c->stages.size(); ++k) {
+    if (c->stages[k].type != T_E) continue;
+    int j = k - 1;   // the backward goes on through the stages before this one
+    bool between = false;
+    for (; j >= 0 && c->stages[j].type != T_E; --j) between = between || (c->stages[j].type != T_G && c->stages[j].type != T_S);
+    c->stages[k].beside = j < 0 || between || (int)c->stages[j].osf.h.size() <= kSmCount;
+  }
+}
+
 // Pointers of the node table for the current structure (present processors), stage lists and launch lists.
 mg_status build_tables(mg_console* c) {
   if (c->is_graph) return build_graph_tables(c);
@@ -1352,6 +1372,7 @@ mg_status build_tables(mg_console* c) {
       c->stages.push_back(st);
     }
   if (join_fir_lists(c) != MG_OK) return MG_ERR_CUDA;
+  adjoint_rule(c);
   // scratch pointers changed with grouping: re-upload the node table
   if (attach_dyn_maps(c) != MG_OK || upload(c, c->hpd, &c->d_procs) != MG_OK) return MG_ERR_CUDA;
   if (upload_procs(c, c->all_present) || upload_procs(c, c->all_lti_present)) return MG_ERR_CUDA;
@@ -1479,6 +1500,7 @@ mg_status build_graph_tables(mg_console* c) {
     c->stages.push_back(st);
   }
   if (join_fir_lists(c) != MG_OK) return MG_ERR_CUDA;
+  adjoint_rule(c);
   if (attach_dyn_maps(c) != MG_OK || upload(c, c->hpd, &c->d_procs) != MG_OK) return MG_ERR_CUDA;
   if (upload_procs(c, c->all_present) || upload_procs(c, c->all_lti_present)) return MG_ERR_CUDA;
   return MG_OK;
