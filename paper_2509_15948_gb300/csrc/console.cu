@@ -609,8 +609,9 @@ struct StageScope {
   ~StageScope() { c->cur_stage = prev; }
 };
 
+// One timed entry of a family; kernels: how many f launches (launches_per_step).
 template <class F>
-void run(mg_console* c, int fam, F&& f) {
+void run(mg_console* c, int fam, F&& f, int kernels = 1) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (c->profiling) {
     if (c->ev_next + 2 > c->ev_pool.size()) {
@@ -625,7 +626,7 @@ void run(mg_console* c, int fam, F&& f) {
     cudaEventRecordWithFlags(e0, c->stream, c->capturing ? cudaEventRecordExternal : cudaEventRecordDefault);
   }
   f();
-  ++c->launches;
+  c->launches += kernels;
   if (c->debug_sync && !c->capturing) {
     // diagnostic mode: wait for every launch and report the first one that fails
     const cudaError_t e = cudaStreamSynchronize(c->stream);
@@ -673,13 +674,13 @@ void run_sized(mg_console* c, int fam, const ItemList& L, F&& f) {
   }
 }
 template <class F>
-void run_procs(mg_console* c, int fam, const ProcList& L, F&& f) {
+void run_procs(mg_console* c, int fam, const ProcList& L, F&& f, int kernels = 1) {
   if (L.h.empty()) return;
   if (!c->per_node) {
-    run(c, fam, [&] { f(L.d, (int)L.h.size()); });
+    run(c, fam, [&] { f(L.d, (int)L.h.size()); }, kernels);
     return;
   }
-  for (size_t i = 0; i < L.h.size(); ++i) run(c, fam, [&] { f(L.d + i, 1); });
+  for (size_t i = 0; i < L.h.size(); ++i) run(c, fam, [&] { f(L.d + i, 1); }, kernels);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
@@ -835,7 +836,7 @@ void stage_backward(mg_console* c, const LaunchCtx& x, Stage& s) {
     case T_E: {
       run_items(c, F_EQ_OS_BWD, s.osf, [&](const Item* it, int n) { launch_eq_os_bwd(x, it, n); });
       const LaunchCtx y = s.beside && c->capturing ? fork(c, x, T_E, c->adj_pending) : x;   // see adjoint_rule
-      run_procs(c, F_FIR_ADJ, s.procs, [&](const int* p, int n) { launch_eq_dh_reduce(y, p, n); });
+      run_procs(c, F_FIR_ADJ, s.procs, [&](const int* p, int n) { launch_eq_dh_reduce(y, p, n); }, 2);
       run_procs(c, F_FIR_ADJ, s.procs, [&](const int* p, int n) { launch_eq_fir_adj(y, p, n); });
       break;
     }
@@ -918,7 +919,7 @@ void backward_pass(mg_console* c, const LaunchCtx& x) {
     run_items(c, F_LOSS_GATHER, c->gather_items,
               [&](const Item* it, int n) { launch_loss_gather(x, c->d_songs, c->d_res, c->nres, it, n); });
   }
-  run(c, F_MISC, [&] { cudaMemsetAsync(c->d_grads, 0, sizeof(float) * c->nparams, c->stream); });
+  run(c, F_MISC, [&] { cudaMemsetAsync(c->d_grads, 0, sizeof(float) * c->nparams, c->stream); }, 0);
   if (c->is_graph) {
     // per schedule step in reverse: the adjoint sums, then the step's processors
     for (int k = (int)c->gstep_type.size() - 1; k >= 0; --k) {
@@ -3114,7 +3115,7 @@ mg_status mg_set_score_mode(mg_console* c, int32_t mode) {
 mg_status mg_adam_step(mg_console* c, float lr, float beta1, float beta2, float eps, float weight_decay) {
   if (!c) return MG_ERR_INVALID;
   launch_set_hyper(c->stream, c->d_hyper, 0, lr, beta1, beta2, eps, weight_decay, 1);
-  run(c, F_ADAM, [&] { launch_adam2(c->stream, c->d_hyper, c->d_step, c->d_params, c->d_grads, c->d_m, c->d_v, c->nparams); });
+  run(c, F_ADAM, [&] { launch_adam2(c->stream, c->d_hyper, c->d_step, c->d_params, c->d_grads, c->d_m, c->d_v, c->nparams); }, 2);
   c->fwd_valid = false;
   c->score_keep.valid = false;
   CK(cudaGetLastError());
@@ -3139,7 +3140,7 @@ mg_status mg_train_step(mg_console* c, float lr, float beta1, float beta2, float
     render(c, x);
     loss_forward(c, x, 1, d_losses, nullptr, 0);
     backward_pass(c, x);
-    run(c, F_ADAM, [&] { launch_adam2(c->stream, c->d_hyper, c->d_step, c->d_params, c->d_grads, c->d_m, c->d_v, c->nparams); });
+    run(c, F_ADAM, [&] { launch_adam2(c->stream, c->d_hyper, c->d_step, c->d_params, c->d_grads, c->d_m, c->d_v, c->nparams); }, 2);
     c->fwd_valid = false;
     c->score_keep.valid = false;
     CK(cudaGetLastError());
@@ -3161,9 +3162,9 @@ mg_status mg_train_step(mg_console* c, float lr, float beta1, float beta2, float
     render(c, x);
     loss_forward(c, x, 1, d_losses, nullptr, 0);
     backward_pass(c, x);
-    run(c, F_ADAM, [&] { launch_adam2(c->stream, c->d_hyper, c->d_step, c->d_params, c->d_grads, c->d_m, c->d_v, c->nparams); });
+    run(c, F_ADAM, [&] { launch_adam2(c->stream, c->d_hyper, c->d_step, c->d_params, c->d_grads, c->d_m, c->d_v, c->nparams); }, 2);
     c->capturing = false;
-    c->launches_step = c->launches;
+    c->launches_step = c->launches + 1;   // and the hyperparameters before the graph
     CK(cudaStreamEndCapture(c->stream, &g));
     CK(cudaGraphInstantiate(&c->graph, g, 0));
     cudaGraphDestroy(g);
