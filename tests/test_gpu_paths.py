@@ -127,3 +127,38 @@ def test_side_streams_against_one_stream(retain):
         out[-1] += [con.get_params().cpu().numpy()]
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("drop", ["", "s", "g"])
+def test_gradients_of_pairs_beside_single_nodes(drop):
+    """The console of the test before, pairs and single nodes side by side: gradients against the FP64 oracle under the same
+    mask (a masked processor's gradients are zero, as a pruned one's read), and the adjoint that every imager writes against
+    its closed form from the adjoint that it reads, within 16 roundings of the summed magnitudes."""
+    import torch
+    from tests.cases import grad_groups, rel_l2
+    case = make_case([W.SongLayout(3, 1, [0, 0, -1], 9001)], types="sg", seed=23)
+    keep = np.ones(len(case.ptypes), np.uint8)
+    for k, i in enumerate(i for i, t in enumerate(case.ptypes) if t == drop):
+        keep[i] = k % 2
+    x = torch.tensor(np.asarray(case.params, np.float64), requires_grad=True)
+    sum(r["total"] for r in case.oracle.forward(x, mask=keep, alpha_p=1e-3)).backward()
+    con = gpu_console(case)
+    if drop:
+        con.prune(keep)
+    con.set_alpha_p(1e-3)
+    con.set_params(case.params)
+    con.forward_loss()
+    con.backward()
+    got = con.get_grads().cpu().numpy()
+    for name, idx in grad_groups(case).items():
+        assert rel_l2(got[idx], x.grad.numpy()[idx]) <= 1e-3, name
+    q = case.params[case.oracle.n_proc_params:].astype(np.float64)
+    for p in case.oracle.procs:
+        if p.type != "s" or not keep[p.index]:
+            continue
+        g, du = con.debug_read(p.index, 5, (2, 9001)).astype(np.float64), con.debug_read(p.index, 3, (2, 9001))
+        w, e = 1.0 / (1.0 + np.exp(-q[p.index])), np.exp(np.float64(case.params[p.offset]))
+        mid, side = 0.5 * w * (g[0] + g[1]), 0.5 * w * e * (g[0] - g[1])
+        want = np.stack([(1 - w) * g[0] + mid + side, (1 - w) * g[1] + mid - side])
+        big = (1 - w) * np.abs(g) + 0.5 * w * (1 + e) * np.abs(g).sum(0)
+        assert (np.abs(du - want) <= 16 * 2.0 ** -24 * big).all(), p.index
