@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
   }
 }
 
-// Channel scales of one node (one CTA per node): per channel the energy of four consecutive samples out of every
+// Channel scales of one node (one CTA per node and operand): per channel the energy of four consecutive samples out of every
 // 128, and of the taps: every 32nd tap of the reverb's dense FIR, all 20 x 39 nonzero taps c_m of the delay's
 // sparse one (a stride would miss whole 39-tap windows).  The scale s = 1/sqrt(e) brings that energy to one, so
 // both channels of a packed transform sit at the same level up to the sampling error of the estimate; 1 for a
@@ -276,8 +276,7 @@ __global__ void __launch_bounds__(kColThreads, 2) k_col(LaunchCtx c, const Item*
 // operands: kScaleOfInput (u), kScaleOfTaps (in the stereo form the transforms use) and kScaleOfAdjoint (dL/dy) bits, one
 // CTA each.  The strided loads are latency: 1,024 threads fetch 4,096 quads (or taps) at a time, and 256 chains add
 // them in order (loading inside the chains of 256 threads, one operand after the other, took 14-20 us per launch on
-// nodes of 10 s and 42-48 on 60 s; now 7-10
-// and 32).
+// nodes of 10 s and 42-48 on 60 s; now 7-10 and 32).
 __device__ __forceinline__ float unit_scale(float e) {
   if (!(e > 0.f) || !isfinite(e)) return 1.f;
   return 1.f / sqrtf(e);

@@ -9,14 +9,15 @@
 //      chunks between: the same multiply-adds in the same order wherever the walk starts, so the state's bits do not
 //      depend on timing; then publishes the state that leaves its own chunk.  The stage's chunks are listed in rounds
 //      across nodes, so on a batch the previous chunk's state is normally there already; on one song, whose nodes do
-//      not fill the GPU, the chain is a hop per 32 chunks instead of one per chunk (a stage of 16 nodes x 10 s took 83 us forward and
-//      103 us backward, now 28 and 63; 8 nodes x 60 s 420 and 480 us, now 70 and 170),
+//      not fill the GPU, the chain is a hop per 32 chunks instead of one per chunk (launches of 16 nodes x 10 s, timed by
+//      events: 94 us forward and 113 backward before, 46 and 96 with it; 8 nodes x 60 s 478 and 508, 110 and 254),
 //   3. rescans its chunk from that state and applies the gain law (Eqs. 13-16) and Eq. (15), fused with the
 //      dry/wet blend.  The forward's input arrives by TMA (a bulk tensor copy into shared memory, read by both
 //      steps) when the node has a tensor map, else by plain loads with the rescan from L2.
 // The adjoint runs the same way in reverse: lambda[n] = dL/dg[n] + alpha lambda[n+1], chunks in reverse order.
 // Its first step also does the per-sample work that does not depend on lambda (the gain law, its partials,
-// dL/dg and the lambda-free part of du), staged in global memory for the same CTA's last step.  A wait that
+// dL/dg and the lambda-free part of du), kept in shared memory for the same CTA's last step (in global memory for a
+// node without tensor maps).  A wait that
 // runs out (about half a second) sets a host-visible error word and continues with a zero state.
 #include "mg_fft.cuh"
 
@@ -424,7 +425,7 @@ __device__ __forceinline__ float4 load_quad(const float* row, int n, int L) {
 // sum lambda[n] (g[n-1] - x[n]).  With tensor maps of u and dL/dy the chunk of both arrives by TMA: step 1 reads
 // them from shared memory and leaves its part of du over dL/dy there and the mid signal and dL/dg over u; step 3 reads
 // all three back, and du is the only signal written (with dL/dg through global memory a sample cost 32 bytes of HBM
-// instead of 24: 16 nodes x 10 s 97 -> 82 us, 8 nodes x 60 s 256 -> 231).  Without maps u and dL/dy are read from
+// instead of 24: the launches of the header, 16 nodes x 10 s 96 -> 82 us, 8 nodes x 60 s 254 -> 219).  Without maps u and dL/dy are read from
 // global memory, and step 1's part of du and dL/dg go through global memory.  Both steps stream a quad at a time.
 __global__ void __launch_bounds__(kThreads, 3) k_dyn_bwd(LaunchCtx c, const Item* __restrict__ items) {
   extern __shared__ unsigned char dsm[];

@@ -10,7 +10,7 @@
 // the SI-SDR sums of the samples after it.  A per-segment kernel adds the pieces in order and forms the feature
 // differences, a per-song kernel combines the segments (double precision, fixed order).
 // The sums are double (FP64 runs at a 64th of FP32's rate here), so the work has to reach every SM: with one CTA per
-// segment a 19 s song (2 segments) took 4.42 ms + 0.14 ms; with 184 CTAs it is latency of one FFT and 16 samples per
+// segment a 19 s song (2 segments) took 4.42 ms + 0.14 ms; with 104 CTAs it is latency of one FFT and 16 samples per
 // thread.
 #include "mg_fftp.cuh"
 

@@ -153,15 +153,6 @@ __global__ void __launch_bounds__(256) k_dly_fir(LaunchCtx c, const Item* __rest
   }
 }
 
-// One CTA per (node, channel, tap m): exact gradient of the 20 log-magnitudes of c_m, and the Eq. (19)
-// update direction of z_m: sgn(g) + gamma (|z| - 1) z/|z| with
-//   g = sum_q G[q] conj(s'_q(z_hat)),  G[q] = sum_j dL/dh[m D + q + j] c_m[j],
-//   s'_q(z) = (1/D) [w^q (1 - z^D) - D z^{D-1} (1 - z w^q)] / (1 - z w^q)^2   (derivative of Eq. 18),
-// z_hat = z / max(1, |z|).  Near a pole (a = z w^q, |1 - a| < 1e-3) the float quotient cancels, and
-// S = sum_{k=1}^{D-1} k a^{k-1} is evaluated in double (pole_sum).  What bounds the kernel: a block used to wait for
-// the one thread at the pole, whose D dependent double steps took 0.86 ms at D = 4410 (nearly all of the kernel's
-// time on a song of 16 tracks); its closed forms take a few microseconds.
-
 // S(a) = sum_{k=1}^{D-1} k a^{k-1} for a on or inside the unit circle, as D terms would give it in double.
 // With e = 1 - a: D |e| <= 6, the binomial series sum_j (-e)^j (j + 1) C(D, j + 2) (terms fall like (D |e|)^j / j!,
 // largest about 300 times the sum); beyond, (1 - a^{D-1} (1 + (D - 1) e)) / e^2, whose numerator no longer cancels.
@@ -226,10 +217,17 @@ __global__ void __launch_bounds__(64) k_dly_pow(LaunchCtx c, const int* __restri
   if (threadIdx.x < kDlyTaps) out[part] = make_float2((float)(rad[m] * ang[0][m]), (float)(rad[m] * ang[1][m]));
 }
 
+// One CTA per (node, channel, tap m): exact gradient of the 20 log-magnitudes of c_m, and the Eq. (19)
+// update direction of z_m: sgn(g) + gamma (|z| - 1) z/|z| with
+//   g = sum_q G[q] conj(s'_q(z_hat)),  G[q] = sum_j dL/dh[m D + q + j] c_m[j],
+//   s'_q(z) = (1/D) [w^q (1 - z^D) - D z^{D-1} (1 - z w^q)] / (1 - z w^q)^2   (derivative of Eq. 18),
+// z_hat = z / max(1, |z|).  Near a pole (a = z w^q, |1 - a| < 1e-3) the float quotient cancels, and
+// S = sum_{k=1}^{D-1} k a^{k-1} is evaluated in double (pole_sum).  What bounds the kernel: a block used to wait for
+// the one thread at the pole, whose D dependent double steps took 0.86 ms at D = 4410 (nearly all of the kernel's
+// time on a song of 16 tracks); its closed forms take a few microseconds.
 __global__ void __launch_bounds__(256) k_dly_adj(LaunchCtx c, const Item* __restrict__ items) {
   __shared__ float cm[kDlyFir];
   __shared__ float dc[kDlyFir];
-  __shared__ float red[2 * 32];
   __shared__ float gsum[2];
   const Item it = items[blockIdx.x];
   const ProcDev& P = c.procs[it.proc];
@@ -280,7 +278,6 @@ __global__ void __launch_bounds__(256) k_dly_adj(LaunchCtx c, const Item* __rest
     accd[0] += (double)G * sp.x;   // g = sum G conj(s'), accumulated in double (|g| can be far below sum |G s'|)
     accd[1] -= (double)G * sp.y;
   }
-  float acc[2] = {0.f, 0.f};
   {
     // block reduction in double: per-warp shuffles, then one warp over the warp totals
     __shared__ double dred[2][32];
@@ -304,8 +301,6 @@ __global__ void __launch_bounds__(256) k_dly_adj(LaunchCtx c, const Item* __rest
       if (lane == 0) { gsum[0] = (float)a0; gsum[1] = (float)a1; }
     }
     __syncthreads();
-    (void)acc;
-    (void)red;
   }
   if (threadIdx.x == 0) {
     const double zr = pz[0], zi = pz[1];

@@ -15,6 +15,10 @@
 // All resolutions are one launch now, the sums go band by band with a weight for four channels, and the loss terms are one
 // coalesced pass (a 30 s mix: forward 242 -> 203 us, adjoint 190 -> 183 by the last two).  Every sum keeps its order, so the
 // losses and gradients keep their bits.
+// The band buffer is the largest resolution's in every mode.  Where it passes 43 KB (linear bins; 96 bands at n_fft 256, 512
+// at 1,024) one CTA fills an SM in the forward too, which the kernel before, with no buffer there, did not; it is the
+// faster one all the same (events, 30 s mix: 512/2048/8192 linear 490 -> 427 us, 256/1024/4096 with 96 bands 355 -> 271,
+// 1024/2048/8192 with 512 bands 425 -> 332; 2 s: 127 -> 33, 106 -> 25, 124 -> 33).
 #include "mg_fftp.cuh"
 
 namespace mg {

@@ -78,7 +78,7 @@ struct ProcDev {
   float* taps;                             // [2][Nh]
   float* dtaps;                            // [2][Nh]
   float* aux;                              // type scratch (delay: c_m and d_m; reverb: adjoint partials;
-                                           // compressor, noisegate: dL/dg per sample)
+                                           // compressor, noisegate without tensor maps: dL/dg per sample)
   // envelope scans (c, n)
   float* carry;                            // [nchunks] forward state entering each chunk
   unsigned long long* cflag;               // [2][nchunks] chained-scan states leaving each chunk, then the chunks'
